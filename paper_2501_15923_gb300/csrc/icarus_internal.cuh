@@ -156,28 +156,53 @@ template <typename R> __device__ __forceinline__ R rabs(R x) { return x < R(0) ?
 template <typename R> __device__ __forceinline__ R rmax(R a, R b) { return a > b ? a : b; }
 template <typename R> __device__ __forceinline__ R rmin(R a, R b) { return a < b ? a : b; }
 
-// Reciprocal 1/q with four FP64 operations: q = +-m 2^E with m in [1, 2); y ~ 1/m from the
-// single-precision rcp.approx on m's leading 23 bits, r = +-y 2^-E assembled on the integer pipe,
-// then two Newton steps t = 1 - q r, r += r t (Markstein, IBM J. Res. Dev. 34 (1990)): the
-// estimate error e becomes e^2 (~6e-14), then e^4, so only the final rounding remains: within one
-// ulp of the correctly rounded reciprocal (equal to it in about 99.3 % of cases). q outside [2^-1021, 2^1021] in magnitude (zero,
-// subnormal, huge, non-finite) takes the library division.
+// The FP64 pipe is the bound of every FP64 kernel (a warp's FP64 instruction holds an SM's pipe for
+// 16 cycles or more, 64 issue slots), so estimates are carried to 44 bits in single precision and one
+// Newton step in double finishes them.
+// Low 29 mantissa bits of the double with words (., lo) as the single-precision tail of its leading
+// 24 bits read as a float with biased exponent 127 + up: in [0, 2^(up - 23)), truncated to 2^(up - 46)
+__device__ __forceinline__ float mant_tail(unsigned int lo, int up)
+{
+    const int e = (104 + up) << 23;
+    return __fsub_rn(__int_as_float(e | (int)((lo >> 6) & 0x7fffffu)), __int_as_float(e));
+}
+// the double with words hi, yb << 29 plus a single-precision correction c: c scale, |c scale| < 2^22,
+// is rounded to an integer (magic addition) and added to the 64-bit pattern at bit sh
+// (bias: units taken off)
+__device__ __forceinline__ double add_tail(int hi, int yb, float c, float scale, int sh, int bias = 0)
+{
+    const int k = __float_as_int(__fmaf_rn(c, scale, 12582912.f)) - (0x4b400000 + bias);
+    const long long b = (long long)(((unsigned long long)(unsigned int)hi << 32) | (unsigned int)(yb << 29));
+    return __longlong_as_double(b + ((long long)k << sh));
+}
+
+// 1 / m for the double q = +-m 2^(e - 1023), m in [1, 2), as bits of a double with q's sign and
+// exponent negated: rcp.approx on m's leading 24 bits (kept in [1/2, 1), so that the binade is known), its
+// residual 1 - m y in single precision, y (2 - m y) to about 2^-43
+__device__ __forceinline__ double rcp_estimate(int hi, unsigned int lo, unsigned int e)
+{
+    const float mh = __int_as_float((127 << 23) | ((hi & 0xfffff) << 3) | (int)(lo >> 29));
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(mh));
+    y = fmaxf(fminf(y, __int_as_float(0x3f7fffff)), 0.5f);
+    const float r = __fmaf_rn(-mant_tail(lo, 0), y, __fmaf_rn(-mh, y, 1.f));
+    const int yb = __float_as_int(y);
+    const int rhi = (hi & (int)0x80000000) | ((2045 - (int)e) << 20) | ((yb & 0x7fffff) >> 3);
+    return add_tail(rhi, yb, __fmul_rn(y, r), 8796093022208.f, 10);     // c in units of 2^-43
+}
+
+// Reciprocal 1/q with two FP64 operations: the 2^-43 estimate above and one Newton step t = 1 - q r,
+// r += r t (Markstein, IBM J. Res. Dev. 34 (1990)), whose error (the square of the estimate's) is far
+// below the final rounding: within one ulp of the correctly rounded reciprocal. q outside
+// [2^-1021, 2^1020] in magnitude (zero, subnormal, huge, non-finite) takes the library division.
 __device__ __forceinline__ double rcp_nr(double q)
 {
     const int hi = __double2hiint(q);
     const unsigned int lo = (unsigned int)__double2loint(q);
     const unsigned int e = ((unsigned int)hi >> 20) & 0x7ffu;
-    if (e - 2u >= 2043u) return 1.0 / q;
-    const int mb = (127 << 23) | ((hi & 0xfffff) << 3) | (int)(lo >> 29);
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__int_as_float(mb)));
-    const int yb = __float_as_int(y);
-    const int rhi = (hi & (int)0x80000000) | ((((yb >> 23) & 0xff) + 1919 - (int)e) << 20) | ((yb & 0x7fffff) >> 3);
-    double r = __hiloint2double(rhi, yb << 29);
-    double t = fma(-q, r, 1.0);
-    r = fma(r, t, r);
-    t = fma(-q, r, 1.0);
-    return fma(r, t, r);
+    if (e - 2u >= 2042u) return 1.0 / q;
+    const double r = rcp_estimate(hi, lo, e);
+    return fma(r, fma(-q, r, 1.0), r);
 }
 __device__ __forceinline__ double rcp_r(double q) { return rcp_nr(q); }
 __device__ __forceinline__ float rcp_r(float q) { return 1.f / q; }
@@ -243,14 +268,16 @@ template <typename R> __device__ __forceinline__ void prim2cons(const R *w, R *u
     u[B3] = w[7];
 }
 
-// Square root of x >= 0 with five FP64 operations, for the wave speeds inside the Riemann flux.
+// Square root of x >= 0 with two FP64 operations, for the wave speeds inside the Riemann flux.
 // x = m 2^(2k) with m in [1, 4) is split on the integer pipe (exponent halved exactly, so every
 // normal double is in range); y ~ 1/sqrt(m) comes from the single-precision rsqrt.approx (relative
-// error below 2^-22.9) on m's leading 23 bits, and r = y 2^-k is widened back on the integer pipe.
-// Then two Newton corrections of the root with the coupled reciprocal (Markstein, IBM J. Res. Dev.
-// 34 (1990)): s = x r, s += (r / 2)(x - s^2), twice. For an estimate error e the first leaves a
-// relative error of about 1.5 e^2 (~3e-14), the second e times that (~1e-21), so the result is the
-// correctly rounded root but for the final rounding: within one ulp of it, almost always equal.
+// error below 2^-22.9) on m's leading 24 bits, p = m y (kept in [1, 2), so that the binade is known)
+// and its residual m - p^2 in single precision give s = p + (m - p^2) y / 2 to about 2^-43. Then one
+// Newton correction with the coupled reciprocal (Markstein, IBM J. Res. Dev. 34 (1990)):
+// s += (y / 2)(x - s^2), whose error (the estimate's times that of y, about 2^-63) is far below the
+// final rounding: within one ulp of the correctly rounded root, almost always equal. s and y are kept
+// a little low, so that the sum errs downwards: the roots of 4^k (1 - 2^-53), just below a rounding
+// boundary, then come out right.
 // Zero, negative, subnormal and non-finite x take the library sqrt.
 __device__ __forceinline__ double sqrt_nr(double x)
 {
@@ -258,18 +285,18 @@ __device__ __forceinline__ double sqrt_nr(double x)
     const unsigned int lo = (unsigned int)__double2loint(x);
     if ((unsigned int)hi - 0x00100000u >= 0x7fe00000u) return sqrt(x);   // not positive and normal
     const int e = hi >> 20;
-    const int k = (e - 1023) >> 1;
-    const int mb = ((127 + e - 1023 - 2 * k) << 23) | ((hi & 0xfffff) << 3) | (int)(lo >> 29);
+    const int k = (e - 1023) >> 1, odd = (e - 1023) & 1;
+    const float mh = __int_as_float(((127 + odd) << 23) | ((hi & 0xfffff) << 3) | (int)(lo >> 29));
     float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__int_as_float(mb)));
-    const int yb = __float_as_int(y);
-    const int rhi = ((((yb >> 23) & 0xff) - 127 + 1023 - k) << 20) | ((yb & 0x7fffff) >> 3);
-    const int rlo = yb << 29;
-    const double r = __hiloint2double(rhi, rlo);               // ~ 1 / sqrt(x)
-    const double h = __hiloint2double(rhi - (1 << 20), rlo);   // r / 2
-    const double s = x * r;
-    const double s1 = fma(h, fma(-s, s, x), s);
-    return fma(h, fma(-s1, s1, x), s1);
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(mh));
+    const float p = fmaxf(fminf(__fmul_rn(mh, y), __int_as_float(0x3fffffff)), 1.f);
+    const float r = __fadd_rn(__fmaf_rn(-p, p, mh), mant_tail(lo, odd));
+    const int yb = __float_as_int(y), pb = __float_as_int(p);
+    const int phi = ((1023 + k) << 20) | ((pb & 0x7fffff) >> 3);
+    const double s = add_tail(phi, pb, __fmul_rn(r, __fmul_rn(0.5f, y)), 4398046511104.f, 10, 2);   // units of 2^-42
+    const int hb = yb - 3;                                      // y / 2, a little low
+    const double h = __hiloint2double((((hb >> 23) + 895 - k) << 20) | ((hb & 0x7fffff) >> 3), hb << 29);
+    return fma(h, fma(-s, s, x), s);
 }
 
 template <bool NR> __device__ __forceinline__ double root(double x) { return NR ? sqrt_nr(x) : sqrt(x); }
@@ -347,6 +374,28 @@ template <typename R> __device__ __forceinline__ R limiter(int lim, R a, R b)
     if (lim == 0) return abs_bits(a) < abs_bits(b) ? a : b;      // minmod
     R m = rmin(rmin(R(2) * rabs(a), R(2) * rabs(b)), R(0.5) * rabs(a + b));   // MC
     return hi_bits(a) >= 0 ? m : -m;
+}
+
+// half the van Leer slope a b / (a + b) of differences a, b with equal signs, s = a + b != 0, with three
+// FP64 operations after the sum: the product p = a b, q ~ p / s to single precision and r ~ 1 / s to
+// about 2^-43 (the estimate of rcp_nr), then q + (p - q s) r, whose error (q's times r's) is far below
+// the final rounding. Sums and products outside [2^-923, 2^177] and [2^-723, 2^967] (where an
+// exponent could leave the normal range) take the library division.
+__device__ __forceinline__ double vanleer_half(double a, double b, double s)
+{
+    const double p = a * b;
+    const int ph = __double2hiint(p), sh = __double2hiint(s);
+    const unsigned int pl = (unsigned int)__double2loint(p), sl = (unsigned int)__double2loint(s);
+    const unsigned int pe = (unsigned int)ph >> 20, se = ((unsigned int)sh >> 20) & 0x7ffu;   // p >= 0
+    if (pe - 300u > 1690u || se - 100u > 1100u) return p / s;
+    const double r = rcp_estimate(sh, sl, se);
+    const float pm = __int_as_float((127 << 23) | ((ph & 0xfffff) << 3) | (int)(pl >> 29));
+    const float sm = __int_as_float((127 << 23) | ((sh & 0xfffff) << 3) | (int)(sl >> 29));
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(sm));
+    const int qb = __float_as_int(__fmul_rn(pm, y));             // m_p / m_s in (1/2, 2)
+    const double q = __hiloint2double((qb >> 3) + (((int)pe - (int)se + 896) << 20) | (sh & (int)0x80000000), qb << 29);
+    return fma(fma(-q, s, p), r, q);
 }
 
 // HLLD (Miyoshi & Kusano 2005): intermediate states separated by the entropy wave S_M and the
@@ -485,6 +534,54 @@ __device__ __forceinline__ void tvdlf_paired(const float *wl, const float *wr, i
     for (int v = 0; v < NV; ++v) f[v] = 0.5f * (F[v].x + F[v].y) - hc * (u[v].y - u[v].x);
 }
 
+// double-precision TVDLF with the fewest FP64 operations (the FP64 pipe is the bound): with the half
+// velocities h = v_n / 2 and the half speed c = c_max / 2, the combination (F_L + F_R)/2 -
+// c_max (U_R - U_L)/2 of a field carried by v_n is U_L (h_L + h_R) + (U_R - U_L)(h_R - c), two
+// operations after the difference, where the terms small against the flux stay small (no
+// cancellation of U (h + c) against U (h - c)); the B_n B / p_tot terms are added from the halved
+// normal field (exact halvings on the integer pipe). The fast speeds come from rho-scaled sums,
+// c_f^2 rho = (S + sqrt(S^2 - 4 gamma p B_n^2)) / 2 with S = gamma p + B^2, so that 1/rho enters once.
+// About 100 FP64 operations a face where the two sides' fluxes and their combination took 130.
+__device__ __forceinline__ void tvdlf_d(const double *wl, const double *wr, int d, double gamma, double igm1, double irl,
+                                        double irr, double *f)
+{
+    const int n = 1 + d, t1 = d == 0 ? 2 : 1, t2 = d == 2 ? 2 : 3;   // normal and tangential velocity fields
+    double m[2][4], e[2], pt[2], bv[2], cs[2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const double *w = s ? wr : wl;
+        m[s][1] = w[0] * w[1];
+        m[s][2] = w[0] * w[2];
+        m[s][3] = w[0] * w[3];
+        const double mv = fma(m[s][1], w[1], fma(m[s][2], w[2], m[s][3] * w[3]));
+        const double bb = fma(w[5], w[5], fma(w[6], w[6], w[7] * w[7]));
+        bv[s] = fma(w[5], w[1], fma(w[6], w[2], w[7] * w[3]));
+        e[s] = fma(w[4], igm1, half_r(mv + bb));
+        pt[s] = fma(0.5, bb, w[4]);
+        const double a = gamma * w[4], S = a + bb, bn = w[4 + n];
+        const double disc = clamp0_r(fma(S, S, -(quad_r(a) * (bn * bn))));
+        cs[s] = sqrt_nr(half_r(S + sqrt_nr(disc)) * (s ? irr : irl));
+    }
+    const double c = half_r(max_nonneg_r(abs_r(wl[n]) + cs[0], abs_r(wr[n]) + cs[1]));
+    const double hl = half_r(wl[n]), hr = half_r(wr[n]), bl = half_r(wl[4 + n]), br = half_r(wr[4 + n]);
+    const double sv = hl + hr, wv = hr - c;
+    f[RHO] = fma(-c, wr[0] - wl[0], half_r(m[0][n] + m[1][n]));
+    f[n] = fma(m[0][n], sv, fma(m[1][n] - m[0][n], wv, half_r(pt[0] + pt[1])));
+    f[n] = fma(-wl[4 + n], bl, fma(-wr[4 + n], br, f[n]));
+    f[t1] = fma(m[0][t1], sv, (m[1][t1] - m[0][t1]) * wv);
+    f[t1] = fma(-wl[4 + t1], bl, fma(-wr[4 + t1], br, f[t1]));
+    f[t2] = fma(m[0][t2], sv, (m[1][t2] - m[0][t2]) * wv);
+    f[t2] = fma(-wl[4 + t2], bl, fma(-wr[4 + t2], br, f[t2]));
+    f[EN] = fma(e[0], sv, (e[1] - e[0]) * wv);
+    f[EN] = fma(pt[0], hl, fma(pt[1], hr, f[EN]));
+    f[EN] = fma(-bv[0], bl, fma(-bv[1], br, f[EN]));
+    f[4 + n] = -c * (wr[4 + n] - wl[4 + n]);            // v_n B_n - B_n v_n is exactly zero
+    f[4 + t1] = fma(wl[4 + t1], sv, (wr[4 + t1] - wl[4 + t1]) * wv);
+    f[4 + t1] = fma(-wl[t1], bl, fma(-wr[t1], br, f[4 + t1]));
+    f[4 + t2] = fma(wl[4 + t2], sv, (wr[4 + t2] - wl[4 + t2]) * wv);
+    f[4 + t2] = fma(-wl[t2], bl, fma(-wr[t2], br, f[4 + t2]));
+}
+
 // TVDLF: (F_L + F_R)/2 - c_max (U_R - U_L)/2; HLL with signal speeds from the fast speeds (flux
 // chosen at run time); HLLD when HD (a separate instantiation, so that the larger solver does not
 // weigh on the registers of the other two)
@@ -497,9 +594,6 @@ __device__ __forceinline__ void riemann(const R *wl, const R *wr, int d, int flu
             return;
         }
     }
-    R ul[NV], ur[NV];
-    prim2cons(wl, ul, igm1);
-    prim2cons(wr, ur, igm1);
     // FP64: 1/rho_L and 1/rho_R from one division, 1 / (rho_L rho_R), while the product stays
     // well inside the normal range (biased exponent test on its bit pattern); two divisions
     // otherwise and in single precision (where a division is cheap)
@@ -519,6 +613,15 @@ __device__ __forceinline__ void riemann(const R *wl, const R *wr, int d, int flu
         irl = R(1) / wl[0];
         irr = R(1) / wr[0];
     }
+    if constexpr (sizeof(R) == 8 && !HD) {
+        if (flux == 0) {
+            tvdlf_d(wl, wr, d, gamma, igm1, irl, irr, f);
+            return;
+        }
+    }
+    R ul[NV], ur[NV];
+    prim2cons(wl, ul, igm1);
+    prim2cons(wr, ur, igm1);
     R cl = fast_speed<R, true>(wl, irl, d, gamma), cr = fast_speed<R, true>(wr, irr, d, gamma);
     R fl[NV], fr[NV];
 #pragma unroll
@@ -546,10 +649,6 @@ __device__ __forceinline__ void riemann(const R *wl, const R *wr, int d, int flu
     if constexpr (HD) {
         (void)flux;
         hlld<R>(wl, wr, ul, ur, fl, fr, cl, cr, d, f);
-    } else if (flux == 0) {
-        const R hc = half_r(max_nonneg_r(abs_r(wl[1 + d]) + cl, abs_r(wr[1 + d]) + cr));
-#pragma unroll
-        for (int v = 0; v < NV; ++v) f[v] = half_r(fl[v] + fr[v]) - hc * (ur[v] - ul[v]);
     } else {
         R sl = rmin(wl[1 + d] - cl, wr[1 + d] - cr);
         R sr = rmax(wl[1 + d] + cl, wr[1 + d] + cr);

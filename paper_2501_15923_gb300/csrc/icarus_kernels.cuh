@@ -320,37 +320,16 @@ __device__ __forceinline__ void flux_tile(const Params &P, const TW *__restrict_
     }
     if (valid) {
         bool half = false;                       // dl holds half the limited slope
-        if (P.limiter == 1 && sizeof(TW) == 8) {
-            // FP64 van Leer 2ab/(a+b) for the eight fields with ONE division: batch inversion of
-            // the eight sums (prefix products, one reciprocal, then peel off; zero sums replaced
-            // by 1); the product stays far inside the double range unless all eight sums are
-            // extreme, in which case the eight divisions are done one by one. dl = ab/(a+b), half
-            // the slope: the factor 2 and the 1/2 of the face extrapolation cancel exactly
+        if (sizeof(TW) == 8 && P.limiter == 1) {
+            // FP64 van Leer: dl = a b / (a + b), half the slope (the factor 2 and the 1/2 of the face
+            // extrapolation cancel exactly), four FP64 operations a field (the batch inversion of the
+            // eight sums took six)
             half = true;
-            TW s[NV], pre[NV];
-            bool ok[NV];
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                s[v] = da[v] + db[v];
-                ok[v] = ((hi_bits(da[v]) ^ hi_bits(db[v])) >= 0) && !is_zero(s[v]);
-                if (!ok[v]) s[v] = TW(1);
-            }
-            pre[0] = s[0];
-#pragma unroll
-            for (int v = 1; v < NV; ++v) pre[v] = pre[v - 1] * s[v];
-            const int ex = (hi_bits(pre[NV - 1]) >> 20) & 0x7ff;     // biased exponent of the product
-            if (ex > 60 && ex < 1990) {
-                TW inv = rcp_r(pre[NV - 1]);
-#pragma unroll
-                for (int v = NV - 1; v > 0; --v) {
-                    const TW iv = inv * pre[v - 1];     // 1 / s[v]
-                    inv = inv * s[v];                   // 1 / (s[0] ... s[v-1])
-                    dl[v] = ok[v] ? da[v] * db[v] * iv : TW(0);
-                }
-                dl[0] = ok[0] ? da[0] * db[0] * inv : TW(0);
-            } else {
-#pragma unroll
-                for (int v = 0; v < NV; ++v) dl[v] = ok[v] ? da[v] * db[v] / s[v] : TW(0);
+                TW s = da[v] + db[v];
+                const bool ok = ((hi_bits(da[v]) ^ hi_bits(db[v])) >= 0) && !is_zero(s);
+                dl[v] = ok ? vanleer_half(da[v], db[v], s) : TW(0);
             }
         } else {
 #pragma unroll
