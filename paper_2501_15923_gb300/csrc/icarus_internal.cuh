@@ -207,6 +207,89 @@ __device__ __forceinline__ double rcp_nr(double q)
 __device__ __forceinline__ double rcp_r(double q) { return rcp_nr(q); }
 __device__ __forceinline__ float rcp_r(float q) { return 1.f / q; }
 
+// the two words of a double through registers that the compiler cannot see through (it turns sign and
+// magnitude operations on a double's bits into FP64 instructions)
+__device__ __forceinline__ void split_d(double x, unsigned int &hi, unsigned int &lo)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "d"(x));
+}
+__device__ __forceinline__ double join_d(unsigned int hi, unsigned int lo)
+{
+    double x;
+    asm("mov.b64 %0, {%1, %2};" : "=d"(x) : "r"(lo), "r"(hi));
+    return x;
+}
+
+// x + y, or x - y with flip = 0x80000000, on the integer pipe, to the bit what the FP64 pipe gives (round
+// to nearest even): the larger magnitude's mantissa with ten guard bits, the other shifted to it with
+// its lost bits jammed into the last, summed in two's complement, normalised and rounded. Sums
+// outside the normal range, of infinities or NaN, or cancelling by more than 2^30 but not to zero take
+// the FP64 addition. About 65 instructions, 32 of the integer pipe's cycles for a warp, beside an FP64
+// instruction's 19 of the FP64 pipe's: worth it where the FP64 pipe is the bound and the others idle.
+// (a call: a branch this short would become a predicated FP64 instruction, which takes its turn on the
+// FP64 pipe with every lane off)
+static __device__ __noinline__ double add_slow(double x, double y, bool minus) { return minus ? x - y : x + y; }
+struct AddI {
+    unsigned int ha, hb;
+    int ea, t;
+    unsigned long long ma, ms;
+    bool sw;
+    __device__ __forceinline__ AddI(unsigned int xh, unsigned int xl, unsigned int yh, unsigned int yl)
+    {
+        const unsigned long long xm = (unsigned long long)(xh & 0x7fffffffu) << 32 | xl,
+                                 ym = (unsigned long long)(yh & 0x7fffffffu) << 32 | yl;
+        sw = xm < ym;
+        ha = sw ? yh : xh; hb = sw ? xh : yh;
+        const unsigned int la = sw ? yl : xl, lb = sw ? xl : yl;
+        ea = (int)((ha >> 20) & 0x7ffu);
+        const int eb = (int)((hb >> 20) & 0x7ffu), d = min(ea - eb, 63);
+        t = (int)(ha ^ hb) >> 31;
+        ma = ((unsigned long long)((ha & 0xfffffu) | (ea ? 0x100000u : 0u)) << 32 | la) << 10;
+        const unsigned long long mb = ((unsigned long long)((hb & 0xfffffu) | (eb ? 0x100000u : 0u)) << 32 | lb) << 10;
+        ms = mb >> d;
+        if ((ms << d) != mb) ms |= 1ull;
+    }
+    // |A| + |B| (t = 0) or |A| - |B| (t = -1) with the sign of hs; the FP64 sum x +- y where that is not covered
+    __device__ __forceinline__ double sum(int t, unsigned int hs, unsigned int hz, double x, double y, bool minus) const
+    {
+        unsigned long long S = ma + ((ms ^ (unsigned long long)(long long)t) + (unsigned long long)(t & 1));
+        const unsigned int sh = (unsigned int)(S >> 32);
+        if (__builtin_expect(S != 0ull && (sh == 0u || (unsigned int)(ea - 64) > 1900u), 0)) return add_slow(x, y, minus);
+        const int n = __clz((int)sh);
+        S <<= n;
+        const unsigned long long m = S >> 11;
+        const unsigned int up = ((unsigned int)S & 0x7ffu) + ((unsigned int)m & 1u) > 0x400u ? 1u : 0u;
+        const unsigned long long r = m + up + ((unsigned long long)((unsigned int)(ea - n) << 20 | (hs & 0x80000000u)) << 32);
+        return S ? join_d((unsigned int)(r >> 32), (unsigned int)r) : join_d(hz & 0x80000000u, 0u);
+    }
+};
+__device__ __forceinline__ double add_i(double x, double y)
+{
+    unsigned int xh, xl, yh, yl;
+    split_d(x, xh, xl);
+    split_d(y, yh, yl);
+    const AddI q(xh, xl, yh, yl);
+    return q.sum(q.t, q.ha, q.ha & q.hb, x, y, false);
+}
+__device__ __forceinline__ double sub_i(double x, double y)
+{
+    unsigned int xh, xl, yh, yl;
+    split_d(x, xh, xl);
+    split_d(y, yh, yl);
+    const AddI q(xh, xl, yh ^ 0x80000000u, yl);
+    return q.sum(q.t, q.ha, q.ha & q.hb, x, y, true);
+}
+// x + y and x - y, sharing the alignment
+__device__ __forceinline__ void add_sub_i(double x, double y, double &s, double &d)
+{
+    unsigned int xh, xl, yh, yl;
+    split_d(x, xh, xl);
+    split_d(y, yh, yl);
+    const AddI q(xh, xl, yh, yl);
+    s = q.sum(q.t, q.ha, q.ha & q.hb, x, y, false);
+    d = q.sum(~q.t, q.sw ? ~q.ha : q.ha, xh & ~yh, x, y, true);
+}
+
 // Exact scalings by 1/2 and 4, |x|, max(x, 0) and the larger of two non-negative values, in
 // double on the integer pipe (exponent field, sign bit, bit-pattern order), since the FP64 pipe is
 // the scarce one; in single precision the plain arithmetic. A scaling is exact whenever its result
@@ -541,7 +624,9 @@ __device__ __forceinline__ void tvdlf_paired(const float *wl, const float *wr, i
 // cancellation of U (h + c) against U (h - c)); the B_n B / p_tot terms are added from the halved
 // normal field (exact halvings on the integer pipe). The fast speeds come from rho-scaled sums,
 // c_f^2 rho = (S + sqrt(S^2 - 4 gamma p B_n^2)) / 2 with S = gamma p + B^2, so that 1/rho enters once.
-// About 100 FP64 operations a face where the two sides' fluxes and their combination took 130.
+// About 100 FP64 operations a face where the two sides' fluxes and their combination took 130; the nine
+// differences U_R - U_L go to the integer pipe (all 20 additions there: the integer pipe becomes the
+// bound, r / theta / phi flux 0.94 / 1.04 / 1.00 ms at 512 x 64 x 128 against 0.91 / 0.98 / 0.94).
 __device__ __forceinline__ void tvdlf_d(const double *wl, const double *wr, int d, double gamma, double igm1, double irl,
                                         double irr, double *f)
 {
@@ -564,21 +649,21 @@ __device__ __forceinline__ void tvdlf_d(const double *wl, const double *wr, int 
     }
     const double c = half_r(max_nonneg_r(abs_r(wl[n]) + cs[0], abs_r(wr[n]) + cs[1]));
     const double hl = half_r(wl[n]), hr = half_r(wr[n]), bl = half_r(wl[4 + n]), br = half_r(wr[4 + n]);
-    const double sv = hl + hr, wv = hr - c;
-    f[RHO] = fma(-c, wr[0] - wl[0], half_r(m[0][n] + m[1][n]));
-    f[n] = fma(m[0][n], sv, fma(m[1][n] - m[0][n], wv, half_r(pt[0] + pt[1])));
+    const double sv = hl + hr, wv = sub_i(hr, c);
+    f[RHO] = fma(-c, sub_i(wr[0], wl[0]), half_r(m[0][n] + m[1][n]));
+    f[n] = fma(m[0][n], sv, fma(sub_i(m[1][n], m[0][n]), wv, half_r(pt[0] + pt[1])));
     f[n] = fma(-wl[4 + n], bl, fma(-wr[4 + n], br, f[n]));
-    f[t1] = fma(m[0][t1], sv, (m[1][t1] - m[0][t1]) * wv);
+    f[t1] = fma(m[0][t1], sv, sub_i(m[1][t1], m[0][t1]) * wv);
     f[t1] = fma(-wl[4 + t1], bl, fma(-wr[4 + t1], br, f[t1]));
-    f[t2] = fma(m[0][t2], sv, (m[1][t2] - m[0][t2]) * wv);
+    f[t2] = fma(m[0][t2], sv, sub_i(m[1][t2], m[0][t2]) * wv);
     f[t2] = fma(-wl[4 + t2], bl, fma(-wr[4 + t2], br, f[t2]));
-    f[EN] = fma(e[0], sv, (e[1] - e[0]) * wv);
+    f[EN] = fma(e[0], sv, sub_i(e[1], e[0]) * wv);
     f[EN] = fma(pt[0], hl, fma(pt[1], hr, f[EN]));
     f[EN] = fma(-bv[0], bl, fma(-bv[1], br, f[EN]));
-    f[4 + n] = -c * (wr[4 + n] - wl[4 + n]);            // v_n B_n - B_n v_n is exactly zero
-    f[4 + t1] = fma(wl[4 + t1], sv, (wr[4 + t1] - wl[4 + t1]) * wv);
+    f[4 + n] = -c * sub_i(wr[4 + n], wl[4 + n]);            // v_n B_n - B_n v_n is exactly zero
+    f[4 + t1] = fma(wl[4 + t1], sv, sub_i(wr[4 + t1], wl[4 + t1]) * wv);
     f[4 + t1] = fma(-wl[t1], bl, fma(-wr[t1], br, f[4 + t1]));
-    f[4 + t2] = fma(wl[4 + t2], sv, (wr[4 + t2] - wl[4 + t2]) * wv);
+    f[4 + t2] = fma(wl[4 + t2], sv, sub_i(wr[4 + t2], wl[4 + t2]) * wv);
     f[4 + t2] = fma(-wl[t2], bl, fma(-wr[t2], br, f[4 + t2]));
 }
 

@@ -243,7 +243,7 @@ template <int D, int BX, int BY, typename TW, bool HD = false, bool GLM = false,
 __device__ __forceinline__ void flux_tile(const Params &P, const TW *__restrict__ W, TW *__restrict__ F,
                                           int bx, int by, int bz, int tx, int ty, TW *sW, TW *sP,
                                           const TP *__restrict__ Psi = nullptr, TW *__restrict__ FP = nullptr,
-                                          TW *sQW = nullptr, TW *sQP = nullptr, TW *sD = nullptr)
+                                          TW *sQW = nullptr, TW *sQP = nullptr)
 {
     constexpr int S = D == 0 ? BX : BY;
     const int ts = D == 0 ? tx : ty;
@@ -284,46 +284,17 @@ __device__ __forceinline__ void flux_tile(const Params &P, const TW *__restrict_
             sQW[sl] = qc;
             sQP[sl] = qc + TW(0.5) * dq;
         }
-        if (sizeof(TW) == 8 && sD) {
-            // FP64: a cell's backward difference is its lower neighbour's forward difference; the
-            // forward differences go through shared memory (the FP64 pipe is the bound, the load
-            // / store path has room), and only the first cell of the tile subtracts its own
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                const TW b = W[v * nt + c], e = W[v * nt + c + st];
-                wc[v] = b;
-                db[v] = e - b;
-                sD[v * sz + sl] = db[v];
-            }
-        } else {
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                TW a = W[v * nt + c - st], b = W[v * nt + c], e = W[v * nt + c + st];
-                wc[v] = b;
-                da[v] = b - a;
-                db[v] = e - b;
-            }
+        for (int v = 0; v < NV; ++v) {
+            TW a = W[v * nt + c - st], b = W[v * nt + c], e = W[v * nt + c + st];
+            wc[v] = b;
+            da[v] = b - a;
+            db[v] = e - b;
         }
-    }
-    if (sizeof(TW) == 8 && sD) {
-        __syncthreads();                             // every thread: the forward differences are in sD
-        if (valid) {
-            const int pn = D == 0 ? sl - 1 : sl - BX;    // the neighbour one cell below along D
-            if (ts > 0) {
-#pragma unroll
-                for (int v = 0; v < NV; ++v) da[v] = sD[v * sz + pn];
-            } else {
-#pragma unroll
-                for (int v = 0; v < NV; ++v) da[v] = wc[v] - W[v * nt + c - st];
-            }
-        }
-    }
-    if (valid) {
         bool half = false;                       // dl holds half the limited slope
         if (sizeof(TW) == 8 && P.limiter == 1) {
             // FP64 van Leer: dl = a b / (a + b), half the slope (the factor 2 and the 1/2 of the face
-            // extrapolation cancel exactly), four FP64 operations a field (the batch inversion of the
-            // eight sums took six)
+            // extrapolation cancel exactly)
             half = true;
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
@@ -373,48 +344,102 @@ __device__ __forceinline__ void flux_tile(const Params &P, const TW *__restrict_
     }
 }
 
+// The FP64 flux tile (TVDLF / HLL). The FP64 pipe bounds it (a warp's instruction takes 19 cycles of an
+// SM's pipe; the other pipes idled), so what can run elsewhere does: the differences, slope sums and
+// face values are additions on the integer pipe (add_i, to the bit the FP64 result), which leaves
+// three FP64 operations a field, 115 a face instead of 155. The reconstruction is a loop over the
+// fields, one field's stencil in registers at a time, both face states through shared memory:
+// unrolled over the eight fields the integer code does not fit the instruction cache (r flux 1.35 ms
+// against 1.03 for the same additions). r / theta / phi flux at 512 x 64 x 128: 1.30 / 1.33 / 1.27 ->
+// 0.91 / 0.98 / 0.94 ms, FP64 pipe saturated with the integer pipe close behind.
+template <int D, int BX, int BY>
+__device__ __forceinline__ void flux_tile_d(const Params &P, const double *__restrict__ W, double *__restrict__ F, int bx,
+                                            int by, int bz, int tx, int ty, double *sL, double *sU)
+{
+    constexpr int S = D == 0 ? BX : BY;
+    const int ts = D == 0 ? tx : ty;
+    const int s = (D == 0 ? bx : by) * (S - 1) - 1 + ts;
+    const int i = D == 0 ? s : bx * BX + tx, j = D == 0 ? by * BY + ty : (D == 1 ? s : bz), k = D == 2 ? s : bz;
+    const bool valid = (D == 0 ? j < P.n2 : i < P.n1) && s <= (D == 0 ? P.n1 : (D == 1 ? P.n2 : P.n3));
+    const long long nt = P.nt, st = D == 0 ? 1 : (D == 1 ? (long long)P.p1 : (long long)P.p1 * P.p2);
+    const int sl = ty * BX + tx, sz = BX * BY;
+    const double *w = W + (valid ? cidx(P, i, j, k) : 0);
+    if (valid) {
+        double a = w[-st], b = w[0], e = w[st];
+#pragma unroll 1
+        for (int v = 0; v < NV; ++v) {
+            const double da = sub_i(b, a), db = sub_i(e, b), wc = b;
+            if (v + 1 < NV) { const double *q = w + (v + 1) * nt; a = q[-st]; b = q[0]; e = q[st]; }
+            double h = 0.0, lo, up;                              // h: half the limited slope
+            if (P.limiter == 1) {
+                if ((hi_bits(da) ^ hi_bits(db)) >= 0 && !is_zero(da) && !is_zero(db)) h = vanleer_half(da, db, add_i(da, db));
+            } else h = half_r(limiter<double>(P.limiter, da, db));
+            add_sub_i(wc, h, up, lo);
+            sL[v * sz + sl] = lo;
+            sU[v * sz + sl] = up;
+        }
+    }
+    if constexpr (D == 0) __syncwarp();
+    else __syncthreads();
+    if (valid && ts > 0 && s >= 0) {
+        double wl[NV], wr[NV], f[NV];
+        const int pl = D == 0 ? sl - 1 : sl - BX;              // the neighbour one cell below along D
+#pragma unroll
+        for (int v = 0; v < NV; ++v) { wl[v] = sU[v * sz + pl]; wr[v] = sL[v * sz + sl]; }
+        if (not_positive(wl[0]) || not_positive(wr[0]) || not_positive(wl[4]) || not_positive(wr[4])) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) { wl[v] = w[v * nt - st]; wr[v] = w[v * nt]; }
+        }
+        riemann<double>(wl, wr, D, P.flux, P.ph.gamma, P.ph.igm1, f);
+        long long fi, fs;
+        if (D == 0) { fi = ((long long)k * P.n2 + j) * (P.n1 + 1) + s; fs = (long long)P.n3 * P.n2 * (P.n1 + 1); }
+        else if (D == 1) { fi = ((long long)k * (P.n2 + 1) + s) * P.n1 + i; fs = (long long)P.n3 * (P.n2 + 1) * P.n1; }
+        else { fi = ((long long)s * P.n2 + j) * P.n1 + i; fs = (long long)(P.n3 + 1) * P.n2 * P.n1; }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) F[v * fs + fi] = f[v];
+    }
+}
+
 // number of tiles of a BX x BY flux tile along each launch axis
 template <int D, int BX, int BY> __host__ __device__ inline void flux_tiles(const Params &P, int &nx, int &ny, int &nz)
 {
-    if (D == 0) { nx = (P.n1 + 1 + BX - 2) / (BX - 1); ny = (P.n2 + BY - 1) / BY; nz = P.n3; }
-    else if (D == 1) { nx = (P.n1 + BX - 1) / BX; ny = (P.n2 + 1 + BY - 2) / (BY - 1); nz = P.n3; }
+    if constexpr (D == 0) { nx = (P.n1 + 1 + BX - 2) / (BX - 1); ny = (P.n2 + BY - 1) / BY; nz = P.n3; }
+    else if constexpr (D == 1) { nx = (P.n1 + BX - 1) / BX; ny = (P.n2 + 1 + BY - 2) / (BY - 1); nz = P.n3; }
     else { nx = (P.n1 + BX - 1) / BX; ny = (P.n3 + 1 + BY - 2) / (BY - 1); nz = P.n2; }
 }
 
-template <int D> struct FluxShape {
-    static constexpr int BX = D == 0 ? 128 : 16;
-    static constexpr int BY = D == 0 ? 1 : 16;
-};
-
-// resident blocks per SM the TVDLF / HLL flux kernels are compiled for. FP64: at most 85 registers,
-// so that 3 blocks of 256 threads (6 of 128) fit in the register file instead of 2 (5) at the 88
-// the compiler takes unasked; the FP64 pipe is their bound, and more warps keep it busier. Single
-// precision: at most 40 registers (6 blocks of 256, 12 of 128; a few bytes of spills) instead of
-// 48, measured 3-7 % faster per flux kernel (issue-bound, latency-limited at 53-56 % warps
-// active). No constraint for the HLLD instantiations.
-template <int D, typename TW, bool HD> struct FluxMinBlocks {
-    static constexpr int value = (sizeof(TW) == 8 && !HD) ? (D == 0 ? 6 : 3) : (!HD ? (D == 0 ? 12 : 6) : 1);
+// Tile shape and resident blocks per SM. FP64 (TVDLF / HLL): the FP64 and integer pipes are the bound,
+// so small blocks of 128 threads, which drift apart and keep both busy: r faces along the 32 lanes of a
+// warp (no block barrier), theta / phi faces in tiles of 8 x 16 (16 x 16: 1.08 / 1.05 ms against 0.98 /
+// 0.94 at 512 x 64 x 128); six blocks at 80 registers (five: 1.01 against 0.94 ms). Single precision: 40
+// registers (6 blocks of 256, 12 of 128; a few bytes of spills) instead of 48, measured 3-7 % faster
+// per flux kernel (issue-bound, latency-limited at 53-56 % warps active). No constraint for HLLD.
+template <int D, typename TW, bool HD> struct FluxShape {
+    static constexpr bool d = sizeof(TW) == 8 && !HD;
+    static constexpr int BX = D == 0 ? (d ? 32 : 128) : (d ? 8 : 16);
+    static constexpr int BY = D == 0 ? (d ? 4 : 1) : 16;
+    static constexpr int MINB = d ? 6 : (!HD ? (D == 0 ? 12 : 6) : 1);
 };
 
 template <int D, typename TW, bool HD = false>
-__global__ void __launch_bounds__(FluxShape<D>::BX * FluxShape<D>::BY, FluxMinBlocks<D, TW, HD>::value)
+__global__ void __launch_bounds__(FluxShape<D, TW, HD>::BX * FluxShape<D, TW, HD>::BY, FluxShape<D, TW, HD>::MINB)
 k_flux(Params P, const TW *__restrict__ W, TW *__restrict__ F)
 {
-    constexpr int BX = FluxShape<D>::BX, BY = FluxShape<D>::BY;
+    constexpr int BX = FluxShape<D, TW, HD>::BX, BY = FluxShape<D, TW, HD>::BY;
     __shared__ TW sW[NV * BY * BX];
     __shared__ TW sP[NV * BY * BX];
-    __shared__ TW sD[sizeof(TW) == 8 && !HD ? NV * BY * BX : 1];   // FP64: forward differences
-    flux_tile<D, BX, BY, TW, HD, false, TW>(P, W, F, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, threadIdx.y, sW,
-                                            sP, nullptr, nullptr, nullptr, nullptr,
-                                            sizeof(TW) == 8 && !HD ? sD : nullptr);
+    if constexpr (FluxShape<D, TW, HD>::d)
+        flux_tile_d<D, BX, BY>(P, W, F, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, threadIdx.y, sW, sP);
+    else
+        flux_tile<D, BX, BY, TW, HD, false, TW>(P, W, F, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, threadIdx.y, sW, sP);
 }
 
 // the same with the GLM face step (psi of type TP, its face fluxes into FP)
 template <int D, typename TW, bool HD, typename TP>
-__global__ void __launch_bounds__(FluxShape<D>::BX * FluxShape<D>::BY)
+__global__ void __launch_bounds__(FluxShape<D, TW, true>::BX * FluxShape<D, TW, true>::BY)
 k_flux_glm(Params P, const TW *__restrict__ W, TW *__restrict__ F, const TP *__restrict__ Psi, TW *__restrict__ FP)
 {
-    constexpr int BX = FluxShape<D>::BX, BY = FluxShape<D>::BY;
+    constexpr int BX = FluxShape<D, TW, true>::BX, BY = FluxShape<D, TW, true>::BY;
     __shared__ TW sW[NV * BY * BX];
     __shared__ TW sP[NV * BY * BX];
     __shared__ TW sQW[BY * BX];
@@ -1519,9 +1544,16 @@ template <typename TS, typename TW> struct Launch {
     }
     template <bool HD> static void flux_dir_t(const Params &P, int dir, const TW *w, TW *F, cudaStream_t s)
     {
-        if (dir == 0) k_flux<0, TW, HD><<<dim3(cdiv(P.n1 + 1, 127), P.n2, P.n3), dim3(128, 1), 0, s>>>(P, w, F);
-        else if (dir == 1) k_flux<1, TW, HD><<<dim3(cdiv(P.n1, 16), cdiv(P.n2 + 1, 15), P.n3), dim3(16, 16), 0, s>>>(P, w, F);
-        else k_flux<2, TW, HD><<<dim3(cdiv(P.n1, 16), cdiv(P.n3 + 1, 15), P.n2), dim3(16, 16), 0, s>>>(P, w, F);
+        if (dir == 0) flux_launch<0, HD>(P, w, F, s);
+        else if (dir == 1) flux_launch<1, HD>(P, w, F, s);
+        else flux_launch<2, HD>(P, w, F, s);
+    }
+    template <int D, bool HD> static void flux_launch(const Params &P, const TW *w, TW *F, cudaStream_t s)
+    {
+        constexpr int BX = FluxShape<D, TW, HD>::BX, BY = FluxShape<D, TW, HD>::BY;
+        int nx, ny, nz;
+        flux_tiles<D, BX, BY>(P, nx, ny, nz);
+        k_flux<D, TW, HD><<<dim3(nx, ny, nz), dim3(BX, BY), 0, s>>>(P, w, F);
     }
     static void flux_dir(const Params &P, int dir, const void *W, void *F, cudaStream_t s)
     {
