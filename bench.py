@@ -282,6 +282,7 @@ def run_batched(ic, torch, args):
         return {"value": cells * steps / (ms * 1e-3) / 1e6, "ms_per_step": ms / steps}
 
     res = {}
+    per_step = ic.icarus_launches_per_step(b.ctx[0])
     for name, mode in (("persistent", ic.ICARUS_BATCH_PERSISTENT), ("phases", ic.ICARUS_BATCH_PHASES),
                        ("concurrent", ic.ICARUS_BATCH_CONCURRENT)):
         b.set_mode(mode)
@@ -289,9 +290,9 @@ def run_batched(ic, torch, args):
             res["phase_tiles"] = b.autotune(2)[0]
         res[name] = timed(b.step)
         res[name]["launches_per_step"] = {ic.ICARUS_BATCH_PERSISTENT: 1, ic.ICARUS_BATCH_PHASES: 18,
-                                          ic.ICARUS_BATCH_CONCURRENT: 17 * len(members)}[mode]
+                                          ic.ICARUS_BATCH_CONCURRENT: per_step * len(members)}[mode]
     res["sequential"] = timed(b.step_sequential)
-    res["sequential"]["launches_per_step"] = len(members) * 17
+    res["sequential"]["launches_per_step"] = len(members) * per_step
     default = "concurrent"      # the library's default form (icarus_batch_set_mode)
     info = b.info()
     dts = sorted(b.time(m)[1] for m in range(len(members)))

@@ -275,7 +275,7 @@ void *icarus_get_stream(icarus_ctx *ctx);
 
 /* Measurement helper: run n_steps steps launching the kernels one by one (no graph) with CUDA
  * events around each launch on the context stream, and return the average duration in ms of one
- * launch of each kernel class: ms[ICARUS_KERNEL_CLASSES] = (ghost fill (3 kernels), flux r,
+ * launch of each kernel class: ms[ICARUS_KERNEL_CLASSES] = (ghost fill, flux r,
  * flux theta, flux phi, div B, update stage 1, update stage 2, probes, fused stage 1, fused
  * stage 2); a class the context does not launch reads 0 (the fused stage kernel replaces the
  * flux, div-B and update kernels of the FP32 and MIXED forms when options.fused = 1; with the
@@ -323,7 +323,7 @@ int icarus_batch_tiles(icarus_batch *b, int m, int *cfg);
  * per-member dt; probes: 18 launches per step whatever the number of members), each over the work
  * items of all members, so that every phase runs with its own register budget; one flux tile shape
  * per direction for the whole ensemble (icarus_batch_autotune times the candidates on the batched
- * launch). ICARUS_BATCH_CONCURRENT: every member's own step (the single solver's kernels, 17 per
+ * launch). ICARUS_BATCH_CONCURRENT: every member's own step (the single solver's kernels, 11 to 13 per
  * member) captured into ONE graph per ensemble step as up to 16 parallel branches (members placed
  * on the least-loaded branch, largest first), so that members' kernels overlap on the GPU; the
  * default (on GB300 the fastest: each kernel keeps the single solver's register budget and reads

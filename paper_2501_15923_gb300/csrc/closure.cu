@@ -1226,7 +1226,7 @@ int icarus_closure_apply(icarus_closure *c, icarus_ctx *ctx)
     c->stream = keep;
     k_apply<<<ccdiv(g.N, 256), 256, 0, s>>>(ctx->P, g, c->y, c->oscale, (double *)ctx->U);
     ctx->ops.prims(ctx->P, ctx->U, ctx->W, s);
-    ctx->ops.fill_ghosts(ctx->P, ctx->U, ctx->W, 1, s);
+    ctx->ops.fill_ghosts(ctx->P, ctx->W, 1, s);
     ctx->ops.cfl(ctx->P, ctx->W, s);
     CCK(cudaGetLastError());
     return ICARUS_OK;
@@ -1270,7 +1270,7 @@ int icarus_restrict(icarus_ctx *fine, icarus_ctx *coarse)
     sc.done = 0;
     CCK(cudaMemcpyAsync(coarse->sc, &sc, sizeof sc, cudaMemcpyHostToDevice, coarse->stream));
     coarse->have_state = true;
-    coarse->ops.fill_ghosts(coarse->P, coarse->U, coarse->W, 1, coarse->stream);
+    coarse->ops.fill_ghosts(coarse->P, coarse->W, 1, coarse->stream);
     coarse->ops.cfl(coarse->P, coarse->W, coarse->stream);
     CCK(cudaGetLastError());
     CCK(cudaStreamSynchronize(coarse->stream));

@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, sizeof(TW) == 4 ? 4 : 2) k_batc
             const Member &M = A.m[m];
             const long long head = M.P.sc->ring_head;
             __syncthreads();
-            for (int p = tid; p < M.P.n_probes; p += blockDim.x) probe_one<TW>(M.P, (const TW *)M.W, p, head);
+            for (int p = tid >> 5; p < M.P.n_probes; p += blockDim.x >> 5) probe_warp<TW>(M.P, (const TW *)M.W, p, head);
             __syncthreads();
             if (tid == 0) M.P.sc->ring_head = head + 1;
         }
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(BATCH_THREADS) k_bp_probe(BatchArgs A)
     const Member &M = stage_member(A, m, sm_member);
     const long long head = M.P.sc->ring_head;
     __syncthreads();
-    for (int p = threadIdx.x; p < M.P.n_probes; p += blockDim.x) probe_one<TW>(M.P, (const TW *)M.W, p, head);
+    for (int p = threadIdx.x >> 5; p < M.P.n_probes; p += blockDim.x >> 5) probe_warp<TW>(M.P, (const TW *)M.W, p, head);
     __syncthreads();
     if (threadIdx.x == 0) M.P.sc->ring_head = head + 1;
 }

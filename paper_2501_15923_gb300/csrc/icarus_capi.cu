@@ -303,9 +303,9 @@ void enqueue_step(icarus_ctx *c, cudaStream_t s)
 {
     const Params &P = c->P;
     if (use_fused_stage(c)) {
-        c->ops.fill_ghosts(P, c->U, c->W, 1, s);
+        c->ops.fill_ghosts(P, c->W, 1, s);
         c->ops.fused_stage(P, 1, c->U, c->W, c->U1, c->W1, s);
-        c->ops.fill_ghosts(P, c->U1, c->W1, 2, s);
+        c->ops.fill_ghosts(P, c->W1, 2, s);
         c->ops.fused_stage(P, 2, c->U1, c->W1, c->U, c->W, s);
         if (P.n_probes > 0) c->ops.probe(P, c->W, s);
         return;
@@ -313,7 +313,7 @@ void enqueue_step(icarus_ctx *c, cudaStream_t s)
     // stage 1: U, W at t  ->  U1, W1 (tracer: rho c in T, c in C  ->  T1, C1, with the stage's mass fluxes)
     // (GLM: psi in Psi -> Psi1 -> Psi, its (B_n, psi) face states after the MHD fluxes)
     const bool tr = c->opts.tracer != 0, glm = P.divb == ICARUS_DIVB_GLM, rf = use_update_rf(c);
-    c->ops.fill_ghosts(P, c->U, c->W, 1, s);
+    c->ops.fill_ghosts(P, c->W, 1, s);
     if (tr) c->ops.tracer_ghost(P, c->C, 1, s);
     if (glm) c->ops.glm_ghost(P, c->Psi, s);
     if (glm) c->ops.fluxes_glm(P, c->W, c->Psi, c->F1, c->F2, c->F3, c->FP1, c->FP2, c->FP3, s);
@@ -325,7 +325,7 @@ void enqueue_step(icarus_ctx *c, cudaStream_t s)
     if (glm) c->ops.glm_update(P, 1, c->Psi, c->Psi1, c->FP1, c->FP2, c->FP3, s);
     if (tr) c->ops.tracer_update(P, 1, c->C, c->F1, c->F2, c->F3, c->T, c->T1, c->U1, c->C1, s);
     // stage 2: U1, W1 at t + dt  ->  U, W (in place), next dt, t += dt
-    c->ops.fill_ghosts(P, c->U1, c->W1, 2, s);
+    c->ops.fill_ghosts(P, c->W1, 2, s);
     if (tr) c->ops.tracer_ghost(P, c->C1, 2, s);
     if (glm) c->ops.glm_ghost(P, c->Psi1, s);
     if (glm) c->ops.fluxes_glm(P, c->W1, c->Psi1, c->F1, c->F2, c->F3, c->FP1, c->FP2, c->FP3, s);
@@ -341,8 +341,8 @@ void enqueue_step(icarus_ctx *c, cudaStream_t s)
 
 int count_launches(const icarus_ctx *c)
 {
-    int per_stage = use_fused_stage(c) ? 3 + 1
-                  : 3 + (use_update_rf(c) ? 2 : 3) + (c->P.divb == 1 || c->P.divb == 3 ? 1 : 0) + 1 +
+    int per_stage = use_fused_stage(c) ? 1 + 1
+                  : 1 + (use_update_rf(c) ? 2 : 3) + (c->P.divb == 1 || c->P.divb == 3 ? 1 : 0) + 1 +
                         (c->opts.tracer ? 2 : 0) +
                         (c->P.divb == ICARUS_DIVB_GLM ? 2 : 0);
     return 2 * per_stage + (c->P.n_probes > 0 ? 1 : 0);
@@ -365,7 +365,7 @@ int build_graph(icarus_ctx *c)
 
 int first_dt(icarus_ctx *c)
 {
-    c->ops.fill_ghosts(c->P, c->U, c->W, 1, c->stream);
+    c->ops.fill_ghosts(c->P, c->W, 1, c->stream);
     c->ops.cfl(c->P, c->W, c->stream);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->stream));
@@ -1008,7 +1008,7 @@ int icarus_time_kernels(icarus_ctx *c, int n_steps, double *ms)
         for (int stage = 1; stage <= 2 && !rc; ++stage) {
             void *Us = stage == 1 ? c->U : c->U1, *Ws = stage == 1 ? c->W : c->W1;
             void *Uo = stage == 1 ? c->U1 : c->U, *Wo = stage == 1 ? c->W1 : c->W;
-            rc |= timed(0, [&] { c->ops.fill_ghosts(P, Us, Ws, stage, s); });
+            rc |= timed(0, [&] { c->ops.fill_ghosts(P, Ws, stage, s); });
             if (fused) {
                 rc |= timed(7 + stage, [&] { c->ops.fused_stage(P, stage, Us, Ws, Uo, Wo, s); });
                 continue;

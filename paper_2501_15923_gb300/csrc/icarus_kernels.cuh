@@ -4,7 +4,7 @@
 //   FP32  : TS = float,  TW = float
 //   MIXED : TS = double, TW = float (update accumulation, dt reduction and the primitive recovery
 //           of the first four radial cells in double)
-// One time step = ghost fill (3 kernels) + face fluxes (3 kernels, one per direction) + div B +
+// One time step = ghost fill + face fluxes (3 kernels, one per direction) + div B +
 // update, twice (SSP-RK2 stages), then the probe kernel. dt and t stay on the device.
 #pragma once
 #include <cstdio>
@@ -70,50 +70,122 @@ __device__ __forceinline__ bool cme_column(const Params &P, double tau, int j, i
 }
 
 // ---------------------------------------------------------------------------------------------
+// time bracket of tau in the map table (clamped outside it): maps m0, m1 and the weight of m1
+__device__ __forceinline__ double map_bracket(const Params &P, double tau, int &m0, int &m1)
+{
+    const int nm = P.n_maps;
+    m0 = m1 = 0;
+    if (!(nm > 1 && tau > P.t_maps[0])) return 0.0;
+    if (tau >= P.t_maps[nm - 1]) { m0 = m1 = nm - 1; return 0.0; }
+    int lo = 0, hi = nm - 1;                        // largest m with t_maps[m] <= tau
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (P.t_maps[mid] <= tau) lo = mid; else hi = mid;
+    }
+    m0 = lo; m1 = lo + 1;
+    const double w = __ddiv_rn(__dsub_rn(tau, P.t_maps[lo]), __dsub_rn(P.t_maps[lo + 1], P.t_maps[lo]));
+    return fmin(fmax(w, 0.0), 1.0);
+}
+
+// boundary values (rho, v_r, p, B_r, B_phi) of the driven column (j, k) at the stage time
+__device__ __forceinline__ void driven_column(const Params &P, int stage, int j, int k, double *q)
+{
+    double tau = P.sc->t;
+    if (stage == 2) tau = __dadd_rn(tau, P.sc->dt);
+    int m0, m1;
+    const double w = map_bracket(P, tau, m0, m1);
+    const long long per = (long long)P.n2 * P.n3, col = (long long)j * P.n3 + k;
+    const int ord[5] = {1, 0, 2, 3, 4};             // maps hold (v_r, rho, p, B_r, B_phi)
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+        const double a = P.maps[((long long)m0 * 5 + ord[f]) * per + col], b = P.maps[((long long)m1 * 5 + ord[f]) * per + col];
+        q[f] = __dadd_rn(__dmul_rn(__dsub_rn(1.0, w), a), __dmul_rn(w, b));
+    }
+    cme_column(P, tau, j, k, q);
+}
+
+// source index of ghost index x along one direction of n cells (continuation, mirror, periodic)
+__device__ __forceinline__ int ghost_source(int bc, int x, int n)
+{
+    if (bc == 1) return x < 0 ? 0 : n - 1;
+    if (bc == 2) return x < 0 ? -x - 1 : 2 * n - 1 - x;
+    return ((x % n) + n) % n;
+}
+
+// every ghost cell of the primitives in one launch, one thread per cell: a ghost along phi, then
+// theta, then r is traced to the interior cell (or driven column) it comes from, so the edges need
+// no earlier pass. (The state's own ghost cells are read by nothing: the primitives carry them.)
+// Bound by latency: one launch of a few microseconds where three in a row (r, theta, phi, with the
+// state's ghosts too) took 23 us on the 60 x 16 x 32 grid and 45 us at 512 x 64 x 128 (now 8 and 19).
+template <typename TW>
+__global__ void __launch_bounds__(128) k_ghost(Params P, TW *__restrict__ W, int stage)
+{
+    const unsigned int nA = 4u * P.p1 * P.p2, nB = 4u * P.p1 * P.n3, nC = 4u * P.n2 * P.n3;
+    unsigned int q = blockIdx.x * blockDim.x + threadIdx.x;
+    int i, j, k;
+    if (q < nC) {                                   // r layers of the interior columns (the longest first)
+        const unsigned int r = q >> 2;
+        k = (int)(r / (unsigned int)P.n2);
+        j = (int)(r - (unsigned int)k * (unsigned int)P.n2);
+        i = (q & 3u) < 2u ? (int)(q & 3u) - NG : P.n1 + (int)(q & 3u) - NG;
+    } else if ((q -= nC) < nA) {                    // phi layers, whole planes
+        const unsigned int r = q / (unsigned int)P.p1, g = r / (unsigned int)P.p2;
+        i = (int)(q - r * (unsigned int)P.p1) - NG;
+        j = (int)(r - g * (unsigned int)P.p2) - NG;
+        k = g < 2u ? (int)g - NG : P.n3 + (int)g - NG;
+    } else if ((q -= nA) < nB) {                    // theta layers of the interior planes
+        const unsigned int r = q / (unsigned int)P.p1;
+        i = (int)(q - r * (unsigned int)P.p1) - NG;
+        k = (int)(r >> 2);
+        j = (r & 3u) < 2u ? (int)(r & 3u) - NG : P.n2 + (int)(r & 3u) - NG;
+    } else return;
+    const long long nt = P.nt, cg = cidx(P, i, j, k);
+    int si = i, sj = j, sk = k;
+    bool flip[3] = {false, false, false};           // mirrored along (r, theta, phi)
+    if (k < 0 || k >= P.n3) { const int bc = P.bc[k < 0 ? 4 : 5]; sk = ghost_source(bc, k, P.n3); flip[2] = bc == 2; }
+    if (j < 0 || j >= P.n2) { const int bc = P.bc[j < 0 ? 2 : 3]; sj = ghost_source(bc, j, P.n2); flip[1] = bc == 2; }
+    TW w[NV];
+    if (i < 0 && P.bc[0] == 3) {
+        double b[5];
+        driven_column(P, stage, sj, sk, b);
+        const long long cm = cidx(P, min(-i - 1, P.n1 - 1), sj, sk);
+        w[0] = (TW)b[0]; w[1] = (TW)b[1]; w[4] = (TW)b[2]; w[5] = (TW)b[3]; w[7] = (TW)b[4];
+        // asymm: v_theta, v_phi, B_theta of the mirror cell with the sign flipped
+        w[2] = -W[2 * nt + cm]; w[3] = -W[3 * nt + cm]; w[6] = -W[6 * nt + cm];
+    } else {
+        if (i < 0 || i >= P.n1) { const int bc = P.bc[i < 0 ? 0 : 1]; si = ghost_source(bc, i, P.n1); flip[0] = bc == 2; }
+        const long long cs = cidx(P, si, sj, sk);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) w[v] = W[v * nt + cs];
+        if (i >= P.n1 && P.bc[1] == 1 && P.geom == 0) {
+            // spherical outer radius: B_r continues as r^-2 (r^2 B_r is copied), so the ghost layer
+            // adds no divergence
+            const double x = P.m.x1c[si + NG] / P.m.x1c[i + NG];
+            w[B1] = (TW)((double)w[B1] * (x * x));
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+        if (flip[d]) { w[M1 + d] = -w[M1 + d]; w[B1 + d] = -w[B1 + d]; }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) W[v * nt + cg] = w[v];
+}
+
+// ---------------------------------------------------------------------------------------------
 // ghost fill along r: inner side driven by the maps (+ CME) or a plain rule, outer side a plain
-// rule. One thread per interior (j, k) column.
+// rule. One thread per interior (j, k) column (the batched forms' phases).
 template <typename TS, typename TW>
-__device__ __forceinline__ void bnd1_col(const Params &P, TS *__restrict__ U, TW *__restrict__ W, int stage, int j, int k,
-                                         int task = -1)
+__device__ __forceinline__ void bnd1_col(const Params &P, TS *__restrict__ U, TW *__restrict__ W, int stage, int j, int k)
 {
     const long long nt = P.nt;
     // inner face
     int bc = P.bc[0];
-    if (task >= NG) {
-        // outer-side layer only
-    } else if (bc == 3) {
-        double tau = P.sc->t;
-        if (stage == 2) tau = __dadd_rn(tau, P.sc->dt);
-        // time bracket (clamped outside the table)
-        int m0 = 0, m1 = 0;
-        double w = 0.0;
-        int nm = P.n_maps;
-        if (nm > 1 && tau > P.t_maps[0]) {
-            if (tau >= P.t_maps[nm - 1]) {
-                m0 = m1 = nm - 1;
-            } else {
-                int m = 0;
-                while (m + 1 < nm - 1 && P.t_maps[m + 1] <= tau) ++m;
-                m0 = m; m1 = m + 1;
-                w = __ddiv_rn(__dsub_rn(tau, P.t_maps[m]), __dsub_rn(P.t_maps[m + 1], P.t_maps[m]));
-                w = fmin(fmax(w, 0.0), 1.0);
-            }
-        }
-        const long long per = (long long)P.n2 * P.n3;
-        const long long col = (long long)j * P.n3 + k;
+    if (bc == 3) {
         double q[5];
-        const int ord[5] = {1, 0, 2, 3, 4};   // maps hold (v_r, rho, p, B_r, B_phi)
-#pragma unroll
-        for (int f = 0; f < 5; ++f) {
-            double a = P.maps[((long long)m0 * 5 + ord[f]) * per + col];
-            double b = P.maps[((long long)m1 * 5 + ord[f]) * per + col];
-            q[f] = __dadd_rn(__dmul_rn(__dsub_rn(1.0, w), a), __dmul_rn(w, b));
-        }
-        cme_column(P, tau, j, k, q);
+        driven_column(P, stage, j, k, q);
         const double igm1 = 1.0 / (P.gamma - 1.0);
 #pragma unroll
         for (int g = 1; g <= NG; ++g) {
-            if (task >= 0 && task != g - 1) continue;
             long long cm_ = cidx(P, g - 1, j, k);
             long long cg = cidx(P, -g, j, k);
             double wg[NV], ug[NV];
@@ -132,7 +204,6 @@ __device__ __forceinline__ void bnd1_col(const Params &P, TS *__restrict__ U, TW
     } else {
 #pragma unroll
         for (int g = 1; g <= NG; ++g) {
-            if (task >= 0 && task != g - 1) continue;
             int src = bc == 1 ? 0 : (bc == 2 ? g - 1 : ((-g % P.n1) + P.n1) % P.n1);
             long long cs = cidx(P, src, j, k), cg = cidx(P, -g, j, k);
 #pragma unroll
@@ -149,7 +220,6 @@ __device__ __forceinline__ void bnd1_col(const Params &P, TS *__restrict__ U, TW
     bc = P.bc[1];
 #pragma unroll
     for (int g = 1; g <= NG; ++g) {
-        if (task >= 0 && task != NG + g - 1) continue;
         int gi = P.n1 - 1 + g;
         int src = bc == 1 ? P.n1 - 1 : (bc == 2 ? P.n1 - g : (gi % P.n1));
         long long cs = cidx(P, src, j, k), cg = cidx(P, gi, j, k);
@@ -174,20 +244,10 @@ __device__ __forceinline__ void bnd1_col(const Params &P, TS *__restrict__ U, TW
     }
 }
 
-template <typename TS, typename TW>
-__global__ void k_bnd1(Params P, TS *__restrict__ U, TW *__restrict__ W, int stage)
-{
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    int k = blockIdx.y;
-    if (j >= P.n2 || k >= P.n3) return;
-    bnd1_col<TS, TW>(P, U, W, stage, j, k, threadIdx.y);     // threadIdx.y: one of the 2 x NG layers
-}
-
 // ghost fill along theta (D = 1) or phi (D = 2) by copy / reflection / periodic images.
 // D = 1 covers every r (ghosts included) and interior phi; D = 2 covers everything.
 template <int D, typename TS, typename TW>
-__device__ __forceinline__ void bnd23_cell(const Params &P, TS *__restrict__ U, TW *__restrict__ W, int ip, int o,
-                                           int task = -1)
+__device__ __forceinline__ void bnd23_cell(const Params &P, TS *__restrict__ U, TW *__restrict__ W, int ip, int o)
 {
     int i = ip - NG;
     const int n = D == 1 ? P.n2 : P.n3;
@@ -197,7 +257,6 @@ __device__ __forceinline__ void bnd23_cell(const Params &P, TS *__restrict__ U, 
         int bc = P.bc[2 * D + side];
 #pragma unroll
         for (int g = 1; g <= NG; ++g) {
-            if (task >= 0 && task != side * NG + g - 1) continue;
             int gi = side == 0 ? -g : n - 1 + g;
             int src;
             if (bc == 1) src = side == 0 ? 0 : n - 1;
@@ -216,17 +275,6 @@ __device__ __forceinline__ void bnd23_cell(const Params &P, TS *__restrict__ U, 
             }
         }
     }
-}
-
-template <int D, typename TS, typename TW>
-__global__ void k_bnd23(Params P, TS *__restrict__ U, TW *__restrict__ W)
-{
-    int ip = blockIdx.x * blockDim.x + threadIdx.x;     // padded r index
-    int o = blockIdx.y;                                 // other index
-    if (ip >= P.p1) return;
-    if (D == 1 && o >= P.n3) return;
-    if (D == 2 && o >= P.p2) return;
-    bnd23_cell<D, TS, TW>(P, U, W, ip, o, threadIdx.y);       // threadIdx.y: one of the 2 x NG layers
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1357,19 +1405,8 @@ __global__ void k_init_state(Params P, TS *__restrict__ U, TW *__restrict__ W, d
     int i = (int)(tid % P.n1);
     long long r_ = tid / P.n1;
     int j = (int)(r_ % P.n2), k = (int)(r_ / P.n2);
-    double tau = P.sc->t;
-    int m0 = 0, m1 = 0;
-    double w = 0.0;
-    int nm = P.n_maps;
-    if (nm > 1 && tau > P.t_maps[0]) {
-        if (tau >= P.t_maps[nm - 1]) m0 = m1 = nm - 1;
-        else {
-            int m = 0;
-            while (m + 1 < nm - 1 && P.t_maps[m + 1] <= tau) ++m;
-            m0 = m; m1 = m + 1;
-            w = fmin(fmax((tau - P.t_maps[m]) / (P.t_maps[m + 1] - P.t_maps[m]), 0.0), 1.0);
-        }
-    }
+    int m0, m1;
+    const double w = map_bracket(P, P.sc->t, m0, m1);
     const long long per = (long long)P.n2 * P.n3, col = (long long)j * P.n3 + k;
     double b[5];
     for (int f = 0; f < 5; ++f)
@@ -1424,108 +1461,115 @@ __global__ void k_unpack(Params P, TS *__restrict__ U, const double *__restrict_
 }
 
 // ---------------------------------------------------------------------------------------------
-// probe sampling at the current time: one thread per probe, one block. Positions use only
-// correctly rounded operations in a fixed order; the stencil is found by comparisons against
-// the cell-centre arrays, so the indices do not depend on the arithmetic of the search.
-template <typename TW>
-__device__ __forceinline__ void probe_one(const Params &P, const TW *__restrict__ W, int p, long long head)
+// for A ascending arrays at once (32 samples of each a round, called by a whole warp): the largest q in
+// [0, n[a]) with x[a][q stride] <= v[a]; below[a]: there is none (q = 0)
+template <int A> __device__ __forceinline__ void warp_search(const double *const *x, int stride, const int *size,
+                                                             const double *v, int *q, bool *below)
 {
-    Scalars *sc = P.sc;
-    {
-        const double AU = 1.495978707e11, PI = 3.14159265358979323846, TWO_PI = 2.0 * 3.14159265358979323846;
-        const double tsi = __dmul_rn(sc->t, P.t0);
-        const double *kn = P.traj + (long long)p * P.n_knots * 4;
-        const int K = P.n_knots;
-        int a = 0;
-        double w = 0.0;
-        if (K == 1 || tsi <= kn[0]) { a = 0; w = 0.0; }
-        else if (tsi >= kn[(K - 1) * 4]) { a = K - 2; w = 1.0; }
-        else {
-            int lo = 0, hi = K - 1;              // largest a with kn[a] <= tsi, a <= K-2
-            while (hi - lo > 1) {
-                int mid = (lo + hi) >> 1;
-                if (kn[mid * 4] <= tsi) lo = mid; else hi = mid;
-            }
-            a = lo;
-            w = __ddiv_rn(__dsub_rn(tsi, kn[a * 4]), __dsub_rn(kn[(a + 1) * 4], kn[a * 4]));
-        }
-        const int b = K == 1 ? 0 : a + 1;
-        const double rm = __dadd_rn(kn[a * 4 + 1], __dmul_rn(w, __dsub_rn(kn[b * 4 + 1], kn[a * 4 + 1])));
-        const double lat = __dadd_rn(kn[a * 4 + 2], __dmul_rn(w, __dsub_rn(kn[b * 4 + 2], kn[a * 4 + 2])));
-        const double lon = __dadd_rn(kn[a * 4 + 3], __dmul_rn(w, __dsub_rn(kn[b * 4 + 3], kn[a * 4 + 3])));
-        const double r = __ddiv_rn(rm, AU);
-        const double th = __dsub_rn(PI / 2.0, lat);
-        double ph = __dsub_rn(lon, __dmul_rn(P.omega_si, tsi));
-        ph = __dsub_rn(ph, __dmul_rn(TWO_PI, floor(__ddiv_rn(ph, TWO_PI))));
-        if (ph >= TWO_PI) ph = 0.0;
-        const Metrics &m = P.m;
-        const double *xc = m.x1c + NG, *yc = m.x2c + NG, *zc = m.x3c + NG;
-        // r: estimate from the position, then move to the largest q in [0, n1-2] with xc[q] <= r
-        int n1 = P.n1, n2 = P.n2, n3 = P.n3;
-        int i = 0, j = 0, k;
-        if (n1 > 1) {
-            double est = (r - xc[0]) / (xc[1] - xc[0]);
-            if (xc[1] / xc[0] > 1.0 + 1e-12 && P.geom == 0) est = log(r / xc[0]) / log(xc[1] / xc[0]);
-            i = (int)fmin(fmax(floor(est), 0.0), (double)(n1 - 2));
-            for (int it = 0; it < n1 && i < n1 - 2 && xc[i + 1] <= r; ++it) ++i;
-            for (int it = 0; it < n1 && i > 0 && xc[i] > r; ++it) --i;
-        }
-        if (n2 > 1) {
-            double est = (th - yc[0]) / (yc[1] - yc[0]);
-            j = (int)fmin(fmax(floor(est), 0.0), (double)(n2 - 2));
-            for (int it = 0; it < n2 && j < n2 - 2 && yc[j + 1] <= th; ++it) ++j;
-            for (int it = 0; it < n2 && j > 0 && yc[j] > th; ++it) --j;
-        }
-        double phk;
-        if (zc[0] > ph) { k = n3 - 1; phk = __dsub_rn(zc[n3 - 1], TWO_PI); }
-        else {
-            double est = floor((ph - zc[0]) * m.id3);
-            k = (int)fmin(fmax(est, 0.0), (double)(n3 - 1));
-            for (int it = 0; it < n3 && k < n3 - 1 && zc[k + 1] <= ph; ++it) ++k;
-            for (int it = 0; it < n3 && k > 0 && zc[k] > ph; ++it) --k;
-            phk = zc[k];
-        }
-        double wr = n1 > 1 ? (r - xc[i]) / (xc[i + 1] - xc[i]) : 0.0;
-        double wt = n2 > 1 ? (th - yc[j]) / (yc[j + 1] - yc[j]) : 0.0;
-        double wp = (ph - phk) * m.id3;
-        wr = fmin(fmax(wr, 0.0), 1.0);
-        wt = fmin(fmax(wt, 0.0), 1.0);
-        wp = fmin(fmax(wp, 0.0), 1.0);
-        const int i1 = n1 > 1 ? i + 1 : i, j1 = n2 > 1 ? j + 1 : j, k1 = (k + 1) % n3;
-        double acc[NV];
+    const int lane = threadIdx.x & 31;
+    int n[A], top = 0;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) acc[v] = 0.0;
-        for (int cc = 0; cc < 8; ++cc) {
-            int ci = (cc & 1) ? i1 : i, cj = (cc & 2) ? j1 : j, ck = (cc & 4) ? k1 : k;
-            double f = ((cc & 1) ? wr : 1.0 - wr) * ((cc & 2) ? wt : 1.0 - wt) * ((cc & 4) ? wp : 1.0 - wp);
-            long long c = cidx(P, ci, cj, ck);
+    for (int a = 0; a < A; ++a) { q[a] = 0; n[a] = size[a]; below[a] = false; top = max(top, n[a]); }
+    for (bool first = true; first || top > 1; first = false) {
+        bool le[A];
+        int step[A];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) acc[v] += f * (double)W[v * P.nt + c];
+        for (int a = 0; a < A; ++a) {
+            step[a] = (n[a] + 31) / 32;
+            const int at = lane * step[a];
+            le[a] = at < n[a] && x[a][(long long)(q[a] + at) * stride] <= v[a];
         }
-        const long long slot = head % P.ring_cap;
-        double *q = P.ring + (slot * P.n_probes + p) * IC_NPROBE_REC;
-        q[0] = tsi;
-        q[1] = acc[0] * 1e6;
-        q[2] = acc[1] * 1e5;
-        q[3] = acc[2] * 1e5;
-        q[4] = (acc[3] + P.omega * r * sin(th)) * 1e5;
-        q[5] = acc[5] * P.b0;
-        q[6] = acc[6] * P.b0;
-        q[7] = acc[7] * P.b0;
-        q[8] = acc[4] * P.p0;
-        q[9] = sqrt(acc[5] * acc[5] + acc[6] * acc[6] + acc[7] * acc[7]) * P.b0;
-        q[10] = i; q[11] = j; q[12] = k;
+        top = 0;
+#pragma unroll
+        for (int a = 0; a < A; ++a) {
+            const int c = __popc(__ballot_sync(0xffffffffu, le[a]));
+            if (first) below[a] = c == 0;
+            const int last = max(c, 1) - 1;
+            q[a] += last * step[a];
+            n[a] = min(step[a], n[a] - last * step[a]);
+            top = max(top, n[a]);
+        }
     }
 }
 
+// probe sampling at the current time, one warp per probe. Positions use only correctly rounded
+// operations in a fixed order; the stencil is found by comparisons against the cell-centre arrays, so
+// the indices do not depend on the arithmetic of the search. Bound by the latency of its dependent loads:
+// the three stencil searches share two rounds of 32 samples each and one lane sums each variable, its
+// eight corners loaded together (between events: one thread per probe 23-31 us, a warp 13-17).
 template <typename TW>
-__global__ void k_probe(Params P, const TW *__restrict__ W)
+__device__ __forceinline__ void probe_warp(const Params &P, const TW *__restrict__ W, int p, long long head)
 {
-    const int p = threadIdx.x;
+    const double AU = 1.495978707e11, PI = 3.14159265358979323846, TWO_PI = 2.0 * 3.14159265358979323846;
+    const int lane = threadIdx.x & 31;
+    const double tsi = __dmul_rn(P.sc->t, P.t0);
+    const double *kn = P.traj + (long long)p * P.n_knots * 4;
+    const int K = P.n_knots;
+    int a = 0;
+    double w = 0.0;
+    if (K == 1 || tsi <= kn[0]) { a = 0; w = 0.0; }
+    else if (tsi >= kn[(long long)(K - 1) * 4]) { a = K - 2; w = 1.0; }
+    else {
+        const int sz = K - 1;
+        bool below;
+        warp_search<1>(&kn, 4, &sz, &tsi, &a, &below);   // largest a with kn[a] <= tsi, a <= K-2
+        w = __ddiv_rn(__dsub_rn(tsi, kn[a * 4]), __dsub_rn(kn[(a + 1) * 4], kn[a * 4]));
+    }
+    const int b = K == 1 ? 0 : a + 1;
+    const double rm = __dadd_rn(kn[a * 4 + 1], __dmul_rn(w, __dsub_rn(kn[b * 4 + 1], kn[a * 4 + 1])));
+    const double lat = __dadd_rn(kn[a * 4 + 2], __dmul_rn(w, __dsub_rn(kn[b * 4 + 2], kn[a * 4 + 2])));
+    const double lon = __dadd_rn(kn[a * 4 + 3], __dmul_rn(w, __dsub_rn(kn[b * 4 + 3], kn[a * 4 + 3])));
+    const double r = __ddiv_rn(rm, AU);
+    const double th = __dsub_rn(PI / 2.0, lat);
+    double ph = __dsub_rn(lon, __dmul_rn(P.omega_si, tsi));
+    ph = __dsub_rn(ph, __dmul_rn(TWO_PI, floor(__ddiv_rn(ph, TWO_PI))));
+    if (ph >= TWO_PI) ph = 0.0;
+    const Metrics &m = P.m;
+    const double *xc = m.x1c + NG, *yc = m.x2c + NG, *zc = m.x3c + NG;
+    const int n1 = P.n1, n2 = P.n2, n3 = P.n3;
+    // the largest q in [0, n - 2] with centre q <= the position (0 below the first centre); along phi
+    // below the first centre the last one, a turn back
+    const double *const x[3] = {xc, yc, zc}, v[3] = {r, th, ph};
+    const int size[3] = {max(n1 - 1, 1), max(n2 - 1, 1), n3};
+    int ijk[3];
+    bool below[3];
+    warp_search<3>(x, 1, size, v, ijk, below);
+    const int i = ijk[0], j = ijk[1], k = zc[0] > ph ? n3 - 1 : ijk[2];
+    const double phk = zc[0] > ph ? __dsub_rn(zc[n3 - 1], TWO_PI) : zc[k];
+    double wr = n1 > 1 ? (r - xc[i]) / (xc[i + 1] - xc[i]) : 0.0;
+    double wt = n2 > 1 ? (th - yc[j]) / (yc[j + 1] - yc[j]) : 0.0;
+    double wp = (ph - phk) * m.id3;
+    wr = fmin(fmax(wr, 0.0), 1.0);
+    wt = fmin(fmax(wt, 0.0), 1.0);
+    wp = fmin(fmax(wp, 0.0), 1.0);
+    const int i1 = n1 > 1 ? i + 1 : i, j1 = n2 > 1 ? j + 1 : j, k1 = (k + 1) % n3;
+    double acc = 0.0;                               // lane v < 8: variable v
+    const TW *wv = W + (lane & 7) * P.nt;
+#pragma unroll
+    for (int cc = 0; cc < 8; ++cc) {
+        const double f = ((cc & 1) ? wr : 1.0 - wr) * ((cc & 2) ? wt : 1.0 - wt) * ((cc & 4) ? wp : 1.0 - wp);
+        acc += f * (double)wv[cidx(P, (cc & 1) ? i1 : i, (cc & 2) ? j1 : j, (cc & 4) ? k1 : k)];
+    }
+    const double b1 = __shfl_sync(0xffffffffu, acc, 5), b2 = __shfl_sync(0xffffffffu, acc, 6), b3 = __shfl_sync(0xffffffffu, acc, 7);
+    const long long slot = head % P.ring_cap;
+    double *q = P.ring + (slot * P.n_probes + p) * IC_NPROBE_REC;
+    if (lane == 0) q[1] = acc * 1e6;
+    else if (lane == 1 || lane == 2) q[lane + 1] = acc * 1e5;
+    else if (lane == 3) q[4] = (acc + P.omega * r * sin(th)) * 1e5;
+    else if (lane == 4) q[8] = acc * P.p0;
+    else if (lane <= 7) q[lane] = acc * P.b0;
+    else if (lane == 8) q[0] = tsi;
+    else if (lane == 9) q[9] = sqrt(b1 * b1 + b2 * b2 + b3 * b3) * P.b0;
+    else if (lane == 10) { q[10] = i; q[11] = j; q[12] = k; }
+}
+
+template <typename TW>
+__global__ void __launch_bounds__(1024) k_probe(Params P, const TW *__restrict__ W)
+{
     const long long head = P.sc->ring_head;
-    if (p < P.n_probes) probe_one<TW>(P, W, p, head);
+    for (int p = threadIdx.x >> 5; p < P.n_probes; p += blockDim.x >> 5) probe_warp<TW>(P, W, p, head);
     __syncthreads();
-    if (p == 0) P.sc->ring_head = head + 1;
+    if (threadIdx.x == 0) P.sc->ring_head = head + 1;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1533,14 +1577,10 @@ __global__ void k_probe(Params P, const TW *__restrict__ W)
 static inline unsigned int cdiv(long long a, long long b) { return (unsigned int)((a + b - 1) / b); }
 
 template <typename TS, typename TW> struct Launch {
-    static void fill_ghosts(const Params &P, void *U, void *W, int stage, cudaStream_t s)
+    static void fill_ghosts(const Params &P, void *W, int stage, cudaStream_t s)
     {
-        TS *u = (TS *)U;
-        TW *w = (TW *)W;
-        const dim3 blk(64, 2 * NG);
-        k_bnd1<TS, TW><<<dim3(cdiv(P.n2, 64), P.n3), blk, 0, s>>>(P, u, w, stage);
-        k_bnd23<1, TS, TW><<<dim3(cdiv(P.p1, 64), P.n3), blk, 0, s>>>(P, u, w);
-        k_bnd23<2, TS, TW><<<dim3(cdiv(P.p1, 64), P.p2), blk, 0, s>>>(P, u, w);
+        const long long n = 4LL * P.p1 * P.p2 + 4LL * P.p1 * P.n3 + 4LL * P.n2 * P.n3;
+        k_ghost<TW><<<cdiv(n, 128), 128, 0, s>>>(P, (TW *)W, stage);
     }
     template <bool HD> static void flux_dir_t(const Params &P, int dir, const TW *w, TW *F, cudaStream_t s)
     {
@@ -1624,7 +1664,7 @@ template <typename TS, typename TW> struct Launch {
     }
     static void probe(const Params &P, const void *W, cudaStream_t s)
     {
-        k_probe<TW><<<1, ((P.n_probes + 31) / 32) * 32, 0, s>>>(P, (const TW *)W);
+        k_probe<TW><<<1, 32 * (P.n_probes < 32 ? P.n_probes : 32), 0, s>>>(P, (const TW *)W);
     }
     static void prims(const Params &P, const void *U, void *W, cudaStream_t s)
     {
