@@ -481,6 +481,27 @@ __device__ __forceinline__ double vanleer_half(double a, double b, double s)
     return fma(fma(-q, s, p), r, q);
 }
 
+// half the limited slope in double precision (van Leer: one integer-pipe sum and vanleer_half)
+__device__ __forceinline__ double half_slope(int lim, double a, double b)
+{
+    if (lim != 1) return half_r(limiter<double>(lim, a, b));
+    return (hi_bits(a) ^ hi_bits(b)) >= 0 && !is_zero(a) && !is_zero(b) ? vanleer_half(a, b, add_i(a, b)) : 0.0;
+}
+
+// half the limited slope in single precision. van Leer 2 a b / (a + b) as the product with the hardware
+// reciprocal, which is what the approximate division gives for 2^-126 <= |a + b| < 2^126 (the same bits)
+// without its range handling; above, where 2 a b only stays finite for a slope negligible against a + b,
+// the slope is 0
+__device__ __forceinline__ float half_slope(int lim, float a, float b)
+{
+    if (lim != 1) return 0.5f * limiter<float>(lim, a, b);
+    const float s = a + b;
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s));
+    const float x = 2.f * a * b * r;
+    return 0.5f * ((__float_as_int(a) ^ __float_as_int(b)) >= 0 && s != 0.f ? x : 0.f);
+}
+
 // HLLD (Miyoshi & Kusano 2005): intermediate states separated by the entropy wave S_M and the
 // rotational waves S*_L, S*_R inside S_L = min(u_L, u_R) - max(c_fL, c_fR), S_R = max(u_L, u_R) +
 // max(c_fL, c_fR); the normal field of the intermediate states is the mean of the two faces'; a
@@ -574,12 +595,10 @@ __device__ __forceinline__ void hlld(const R *wl, const R *wr, const R *ul, cons
 // instructions (x = left, y = right): conserved states, fast speeds and physical fluxes of both
 // sides from one instruction stream; the combination (F_L + F_R)/2 - c_max (U_R - U_L)/2 per lane
 __device__ __forceinline__ float2 f2_(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ void tvdlf_paired(const float *wl, const float *wr, int d, float gamma, float igm1, float *f)
+__device__ __forceinline__ void tvdlf_paired(const float2 *w, int d, float gamma, float igm1, float *f)
 {
-    float2 w[NV], u[NV], F[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) w[v] = f2_(wl[v], wr[v]);
-    const float2 h = f2_(0.5f, 0.5f), irho = f2_(1.f / wl[0], 1.f / wr[0]);
+    float2 u[NV], F[NV];
+    const float2 h = f2_(0.5f, 0.5f), irho = f2_(1.f / w[0].x, 1.f / w[0].y);
     u[RHO] = w[0];
     u[M1] = __fmul2_rn(w[0], w[1]);
     u[M2] = __fmul2_rn(w[0], w[2]);
@@ -675,7 +694,10 @@ __device__ __forceinline__ void riemann(const R *wl, const R *wr, int d, int flu
 {
     if constexpr (sizeof(R) == 4 && !HD) {
         if (flux == 0) {
-            tvdlf_paired(wl, wr, d, gamma, igm1, f);
+            float2 w[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) w[v] = f2_(wl[v], wr[v]);
+            tvdlf_paired(w, d, gamma, igm1, f);
             return;
         }
     }

@@ -321,7 +321,7 @@ __device__ __forceinline__ void flux_tile(const Params &P, const TW *__restrict_
     const int sl = ty * BX + tx, sz = BX * BY;
     TW wc[NV], wm[NV];
     TW qc = TW(0), qm = TW(0);
-    TW da[NV], db[NV], dl[NV];
+    TW da[NV], db[NV];
     const long long c = valid ? cidx(P, i, j, k) : 0;
     if (valid) {
         if constexpr (GLM) {
@@ -339,24 +339,9 @@ __device__ __forceinline__ void flux_tile(const Params &P, const TW *__restrict_
             da[v] = b - a;
             db[v] = e - b;
         }
-        bool half = false;                       // dl holds half the limited slope
-        if (sizeof(TW) == 8 && P.limiter == 1) {
-            // FP64 van Leer: dl = a b / (a + b), half the slope (the factor 2 and the 1/2 of the face
-            // extrapolation cancel exactly)
-            half = true;
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                TW s = da[v] + db[v];
-                const bool ok = ((hi_bits(da[v]) ^ hi_bits(db[v])) >= 0) && !is_zero(s);
-                dl[v] = ok ? vanleer_half(da[v], db[v], s) : TW(0);
-            }
-        } else {
-#pragma unroll
-            for (int v = 0; v < NV; ++v) dl[v] = limiter<TW>(P.limiter, da[v], db[v]);
-        }
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-            const TW h = half ? dl[v] : TW(0.5) * dl[v];
+            const TW h = half_slope(P.limiter, da[v], db[v]);
             wm[v] = wc[v] - h;
             sW[v * sz + sl] = wc[v];
             sP[v * sz + sl] = wc[v] + h;
@@ -418,11 +403,8 @@ __device__ __forceinline__ void flux_tile_d(const Params &P, const double *__res
         for (int v = 0; v < NV; ++v) {
             const double da = sub_i(b, a), db = sub_i(e, b), wc = b;
             if (v + 1 < NV) { const double *q = w + (v + 1) * nt; a = q[-st]; b = q[0]; e = q[st]; }
-            double h = 0.0, lo, up;                              // h: half the limited slope
-            if (P.limiter == 1) {
-                if ((hi_bits(da) ^ hi_bits(db)) >= 0 && !is_zero(da) && !is_zero(db)) h = vanleer_half(da, db, add_i(da, db));
-            } else h = half_r(limiter<double>(P.limiter, da, db));
-            add_sub_i(wc, h, up, lo);
+            double lo, up;
+            add_sub_i(wc, half_slope(P.limiter, da, db), up, lo);
             sL[v * sz + sl] = lo;
             sU[v * sz + sl] = up;
         }
@@ -446,6 +428,78 @@ __device__ __forceinline__ void flux_tile_d(const Params &P, const double *__res
 #pragma unroll
         for (int v = 0; v < NV; ++v) F[v * fs + fi] = f[v];
     }
+}
+
+// Single-precision theta / phi faces (TVDLF / HLL): a thread marches along D through a chunk of faces of one
+// column, the columns flattened over (r, other index) so that lanes follow r. Each cell is loaded once,
+// one face ahead (without that the loads' latency is paid at every face: 180-260 us), its backward
+// difference is the previous cell's forward one and its upper face state stays in registers for the
+// next face: no shared memory, no barrier, one reconstruction in L + 1 wasted per chunk of L faces.
+// Bound by instruction issue, 64 % of the slots busy: 340 instructions a face instead of 530 for tiles of 16 x 16 through shared
+// memory; theta / phi 76 / 72 -> 65 / 66 us at 512 x 64 x 128, 22 / 20 -> 16 / 16 at 300 x 33 x 65 (six blocks
+// of 128 per SM at 80 registers; five 68 / 67, seven 75 / 73).
+template <int D>
+__global__ void __launch_bounds__(128, 6)
+k_flux_march(Params P, const float *__restrict__ W, float *__restrict__ F, int L)
+{
+    const unsigned int q = blockIdx.x * 128u + threadIdx.x, n1 = (unsigned int)P.n1, no = D == 1 ? P.n3 : P.n2;
+    if (q >= n1 * no) return;
+    const int o = (int)(q / n1), i = (int)(q - (unsigned int)o * n1), nf = (D == 1 ? P.n2 : P.n3) + 1;
+    const int f0 = blockIdx.y * L, f1 = min(f0 + L, nf);
+    // (field base + 32-bit offset: one address instruction an access; a field has below 2^31 cells and faces)
+    const long long nt = P.nt;
+    const unsigned int st = D == 1 ? (unsigned int)P.p1 : (unsigned int)P.p1 * (unsigned int)P.p2;
+    unsigned int c = (unsigned int)(D == 1 ? cidx(P, i, f0 - 1, o) : cidx(P, i, o, f0 - 1));   // cell below the face
+    const long long fs = D == 1 ? (long long)P.n3 * nf * P.n1 : (long long)nf * P.n2 * P.n1;
+    const unsigned int fst = D == 1 ? n1 : (unsigned int)P.n2 * n1;
+    unsigned int f = D == 1 ? ((unsigned int)o * nf + f0) * n1 + i : ((unsigned int)f0 * P.n2 + o) * n1 + i;
+    float b[NV], d[NV], up[NV], nx[NV];               // the cell above the face, its backward difference; state below
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        const float *w = W + v * nt;
+        const float a = w[c - st], wc = w[c];
+        b[v] = w[c + st];
+        d[v] = b[v] - wc;
+        up[v] = wc + half_slope(P.limiter, wc - a, d[v]);
+        nx[v] = w[c + 2u * st];
+    }
+#pragma unroll 2
+    for (int s = f0; s < f1; ++s) {
+        c += st;                                      // the cell above the face
+        float e8[NV];                                 // loaded a face ahead
+#pragma unroll
+        for (int v = 0; v < NV; ++v) e8[v] = nx[v];
+        if (s + 1 < f1) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) nx[v] = (W + v * nt)[c + 2u * st];
+        }
+        float wr[NV], nu[NV], fl[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const float e = e8[v], de = e - b[v], h = half_slope(P.limiter, d[v], de);
+            wr[v] = b[v] - h;
+            nu[v] = b[v] + h;
+            b[v] = e;
+            d[v] = de;
+        }
+        if (not_positive(up[0]) || not_positive(wr[0]) || not_positive(up[4]) || not_positive(wr[4])) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) { up[v] = (W + v * nt)[c - st]; wr[v] = (W + v * nt)[c]; }
+        }
+        riemann<float>(up, wr, D, P.flux, P.phf.gamma, P.phf.igm1, fl);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) { (F + v * fs)[f] = fl[v]; up[v] = nu[v]; }
+        f += fst;
+    }
+}
+
+// faces a thread marches through: 16, fewer (4 at least) while the chunks do not give every SM 48 warps
+inline int march_length(long long columns, int faces)
+{
+    const long long warps = (columns + 31) / 32, want = (152LL * 48 + warps - 1) / warps;
+    const long long lo = (faces + 15) / 16, hi = (faces + 3) / 4;
+    const long long chunks = want < lo ? lo : (want < hi ? want : hi);
+    return (int)((faces + chunks - 1) / chunks);
 }
 
 // number of tiles of a BX x BY flux tile along each launch axis
@@ -752,18 +806,15 @@ template <typename TW> struct DivFactors {
     }
 };
 
-// the update of one interior cell (i, j, k) from its primitives w, the flux divergence L (in:
-// per field, out: the full residual), div B at its six neighbours, its stage-start state us(v)
-// and (second stage) U^n un(v) (accessors, so that loads sit where they are used): the new state
-// uo and primitives wo (floors applied and counted)
-template <int STAGE, typename TS, typename TW, typename LS, typename LN>
-__device__ __forceinline__ void update_math(const Params &P, int i, int j, int k, const TW *w, TW *L, const TW *dbn,
-                                            LS us, LN un, TS *uo, TW *wo)
+// the sources of one interior cell (i, j, k) from its primitives w and div B at its six neighbours: added
+// to the flux divergence L; lb receives the Linde increment of B (lin: it acts, dt > 0)
+template <typename TW>
+__device__ __forceinline__ void update_sources(const Params &P, int i, int j, int k, const TW *w, TW *L, const TW *dbn,
+                                               bool lin, TW *lb)
 {
     const int ip = i + NG, jp = j + NG;
     const MetricsT<TW> &m = met<TW>(P);
     const PhysT<TW> &ph = phys<TW>(P);
-    const double dt = P.sc->dt;
     if (P.geom == 0) {
         const TW rho = w[0], vr = w[1], vt = w[2], vp = w[3];
         const TW br = w[5], bt = w[6], bp = w[7];
@@ -776,7 +827,7 @@ __device__ __forceinline__ void update_math(const Params &P, int i, int j, int k
         L[M3] -= ((rho * vp * vr - bp * br) + cot * (rho * vp * vt - bp * bt)) * ir;
         L[B2] += (vr * bt - vt * br) * ir;
         L[B3] += ((vr * bp - vp * br) + cot * (vt * bp - vp * bt)) * ir;
-        if (P.omega != 0.0) {
+        if (ph.omega != TW(0)) {
             // co-rotating frame, Omega along the polar axis: centrifugal rho Omega^2 r sin(th)
             // (sin th, cos th, 0), Coriolis 2 rho Omega (v_phi sin th, v_phi cos th,
             // -(v_r sin th + v_th cos th)), work of the centrifugal force in e
@@ -815,8 +866,8 @@ __device__ __forceinline__ void update_math(const Params &P, int i, int j, int k
     }
     // Linde div-B diffusion: increment C_d / (sum_d 1/dx_d^2) grad(div B) per stage;
     // dbn = div B at (i-1, i+1, j-1, j+1, k-1, k+1)
-    TW lb[3] = {TW(0), TW(0), TW(0)};
-    if (P.divb == 1 && dt > 0.0) {
+    lb[0] = lb[1] = lb[2] = TW(0);
+    if (lin) {
         if constexpr (sizeof(TW) == 8) {
             // coefficient times inverse widths from the per-cell table
             lb[0] = (dbn[1] - dbn[0]) * cfv(m, CF_LD0, ip, jp);
@@ -829,6 +880,16 @@ __device__ __forceinline__ void update_math(const Params &P, int i, int j, int k
             lb[2] = coef * (dbn[5] - dbn[4]) * (m.ih2[ip] * m.is3[jp] * m.ig3[k + NG]);
         }
     }
+}
+
+// the new state uo of the cell from its stage-start state us(v), (second stage) U^n un(v) (accessors, so
+// that loads sit where they are used), its residual L and Linde increment lb, and its primitives wo
+// (floors applied and counted)
+template <int STAGE, typename TS, typename TW, typename LS, typename LN>
+__device__ __forceinline__ void update_apply(const Params &P, int i, const TW *w, const TW *L, const TW *lb, double dt, LS us,
+                                             LN un, TS *uo, TW *wo)
+{
+    const PhysT<TW> &ph = phys<TW>(P);
     if constexpr (Prec<TS, TW>::mixed) {
         // MIXED: the increment dt L + (Linde term) is formed in single precision like the fluxes it
         // comes from, and accumulated onto the FP64 state with one exact widening per field; the
@@ -844,7 +905,9 @@ __device__ __forceinline__ void update_math(const Params &P, int i, int j, int k
             else uo[v] = half_r(un(v) + x);
         }
     } else {
-        const TS dts = (TS)dt;
+        TS dts;
+        if constexpr (sizeof(TS) == 4) dts = narrow_d2f(dt);
+        else dts = dt;
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             // the Linde increment exists for e and B only (no addition of a zero for the others);
@@ -887,20 +950,33 @@ __device__ __forceinline__ void update_math(const Params &P, int i, int j, int k
     }
 }
 
+// the update of one interior cell (i, j, k): its sources, then its new state
+template <int STAGE, typename TS, typename TW, typename LS, typename LN>
+__device__ __forceinline__ void update_math(const Params &P, int i, int j, int k, const TW *w, TW *L, const TW *dbn,
+                                            LS us, LN un, TS *uo, TW *wo)
+{
+    const double dt = P.sc->dt;
+    TW lb[3];
+    update_sources<TW>(P, i, j, k, w, L, dbn, P.divb == 1 && __double2hiint(dt) > 0, lb);
+    update_apply<STAGE, TS, TW>(P, i, w, L, lb, dt, us, un, uo, wo);
+}
+
 // update_math of cell (i, j, k) with its state read from and written to the global arrays (U^n is
 // updated in place in the second stage)
 template <int STAGE, typename TS, typename TW>
 __device__ __forceinline__ void update_core(const Params &P, int i, int j, int k, const TW *w, TW *L, const TW *dbn,
                                             const TS *__restrict__ Us, TS *Uo, TW *__restrict__ Wo, TW *wo)
 {
-    const long long nt = P.nt, c = cidx(P, i, j, k);
+    // (field base + 32-bit offset: one address instruction an access; a field has below 2^31 cells)
+    const long long nt = P.nt;
+    const unsigned int c = (unsigned int)cidx(P, i, j, k);
     TS uo[NV];
-    update_math<STAGE, TS, TW>(P, i, j, k, w, L, dbn, [&](int v) { return Us[v * nt + c]; },
-                               [&](int v) { return Uo[v * nt + c]; }, uo, wo);
+    update_math<STAGE, TS, TW>(P, i, j, k, w, L, dbn, [&](int v) { return (Us + v * nt)[c]; },
+                               [&](int v) { return (Uo + v * nt)[c]; }, uo, wo);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-        Uo[v * nt + c] = uo[v];
-        Wo[v * nt + c] = wo[v];
+        (Uo + v * nt)[c] = uo[v];
+        (Wo + v * nt)[c] = wo[v];
     }
 }
 
@@ -1007,6 +1083,10 @@ __host__ __device__ inline long long rf_blocks(const Params &P)
 // its two r fluxes from shared memory and its theta / phi fluxes from the arrays of the separate
 // flux kernels. The arithmetic of each step is that of flux_tile<0> and update_cell. Every
 // thread of the block reaches the barriers (threads past the segment's end only skip the work).
+// Field bases with 32-bit offsets save an address instruction in two (FP32 0.222 / 0.268 -> 0.212 /
+// 0.258 ms per stage). Tried and slower: a lane for two cells with shuffles instead of shared memory (0.42 / 0.53
+// MIXED; with its fluxes and states by asynchronous copies 0.45 / 0.64), a lane for one (0.35 / 0.43), L2
+// prefetches of what the update reads (no change).
 // Measured at 512 x 64 x 128 (four segments of 128 per row, eight resident blocks per SM at 64
 // registers): MIXED step 1.115 -> 1.012 ms, FP32 0.960 -> 0.877 ms against the r-flux kernel +
 // update. Segments of 256 (four blocks per SM) took 1.050 / 0.896 ms, of 64 (sixteen) 1.035 /
@@ -1027,17 +1107,18 @@ k_update_rf(Params P, const TS *__restrict__ Us, const TW *__restrict__ Ws, TS *
     const int seg = (int)(blockIdx.x - row * (unsigned int)ns);
     const int j = (int)(row % (unsigned int)P.n2), k = (int)(row / (unsigned int)P.n2);
     const int i0 = seg * C, nc = min(C, P.n1 - i0);
-    const long long nt = P.nt, c0 = cidx(P, i0, j, k);
+    const long long nt = P.nt;
+    const unsigned int c0 = (unsigned int)cidx(P, i0, j, k);
     for (int q = t; q < nc + 4; q += C) {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) sW[v][q] = Ws[v * nt + c0 - 2 + q];
+        for (int v = 0; v < NV; ++v) sW[v][q] = (Ws + v * nt)[c0 - 2u + q];
     }
     __syncthreads();
     for (int q = t; q < nc + 2; q += C) {          // cell i0 - 1 + q (sW index q + 1)
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             const TW wc = sW[v][q + 1];
-            const TW h = TW(0.5) * limiter<TW>(P.limiter, wc - sW[v][q], sW[v][q + 2] - wc);
+            const TW h = half_slope(P.limiter, wc - sW[v][q], sW[v][q + 2] - wc);
             sL[v][q] = wc - h;
             sU[v][q] = wc + h;
         }
@@ -1060,20 +1141,20 @@ k_update_rf(Params P, const TS *__restrict__ Us, const TW *__restrict__ Ws, TS *
     const int i = i0 + t;
     TW wo[NV];
     if (valid) {
-        const long long c = c0 + t;
-        const long long s2 = (long long)P.n3 * (P.n2 + 1) * P.n1, f2 = ((long long)k * (P.n2 + 1) + j) * P.n1 + i;
-        const long long s3 = (long long)(P.n3 + 1) * P.n2 * P.n1, f3 = ((long long)k * P.n2 + j) * P.n1 + i;
-        const long long o3 = (long long)P.n2 * P.n1;
+        const unsigned int c = c0 + t, n1 = P.n1, n2 = P.n2;
+        const long long s2 = (long long)P.n3 * (P.n2 + 1) * P.n1, s3 = (long long)(P.n3 + 1) * P.n2 * P.n1;
+        const unsigned int f2 = ((unsigned int)k * (n2 + 1u) + (unsigned int)j) * n1 + (unsigned int)i;
+        const unsigned int f3 = ((unsigned int)k * n2 + (unsigned int)j) * n1 + (unsigned int)i, o3 = n2 * n1;
         const DivFactors<TW> dv(met<TW>(P), i + NG, j + NG);
         TW w[NV], L[NV], dbn[7];
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             w[v] = sW[v][t + 2];
-            L[v] = dv.div(sF[v][t], sF[v][t + 1], F2[v * s2 + f2], F2[v * s2 + f2 + P.n1], F3[v * s3 + f3],
-                          F3[v * s3 + f3 + o3]);
+            L[v] = dv.div(sF[v][t], sF[v][t + 1], (F2 + v * s2)[f2], (F2 + v * s2)[f2 + n1], (F3 + v * s3)[f3],
+                          (F3 + v * s3)[f3 + o3]);
         }
         if (P.divb == 1) {
-            const long long q2 = P.p1, q3 = (long long)P.p1 * P.p2;
+            const unsigned int q2 = P.p1, q3 = (unsigned int)P.p1 * (unsigned int)P.p2;
             dbn[0] = divB[c - 1]; dbn[1] = divB[c + 1];
             dbn[2] = divB[c - q2]; dbn[3] = divB[c + q2];
             dbn[4] = divB[c - q3]; dbn[5] = divB[c + q3];
@@ -1085,6 +1166,10 @@ k_update_rf(Params P, const TS *__restrict__ Us, const TW *__restrict__ Ws, TS *
     if (STAGE == 2) finish_dt(P, cfl_block_speed<TW>(P, wo, (valid ? i : 0) + NG, j + NG, valid), 1);
 }
 
+template <typename T> struct Vec2;
+template <> struct Vec2<float> { using t = float2; };
+template <> struct Vec2<double> { using t = double2; };
+
 // FP32 form, n1 even: one thread updates the two cells (i, i+1), i even, of a radial row with
 // two-element vector loads and stores (every array offset of such a pair is even: p1, n1, the
 // field strides and the base addresses are), which halves the memory instructions of this
@@ -1093,10 +1178,6 @@ k_update_rf(Params P, const TS *__restrict__ Us, const TW *__restrict__ Ws, TS *
 // blocks per SM, measured at 512 x 64 x 128: the first stage at three (at most 85 registers, 0.176
 // against 0.189 ms at two), the second, with U^n and the CFL reduction, at two (0.275 against 0.300
 // ms at three)
-template <typename T> struct Vec2;
-template <> struct Vec2<float> { using t = float2; };
-template <> struct Vec2<double> { using t = double2; };
-
 template <int STAGE, typename TS, typename TW>
 __global__ void __launch_bounds__(256, STAGE == 1 ? 3 : 2)
 k_update_pair(Params P, const TS *__restrict__ Us, const TW *__restrict__ Ws, TS *Uo, TW *__restrict__ Wo,
@@ -1590,10 +1671,16 @@ template <typename TS, typename TW> struct Launch {
     }
     template <int D, bool HD> static void flux_launch(const Params &P, const TW *w, TW *F, cudaStream_t s)
     {
-        constexpr int BX = FluxShape<D, TW, HD>::BX, BY = FluxShape<D, TW, HD>::BY;
-        int nx, ny, nz;
-        flux_tiles<D, BX, BY>(P, nx, ny, nz);
-        k_flux<D, TW, HD><<<dim3(nx, ny, nz), dim3(BX, BY), 0, s>>>(P, w, F);
+        if constexpr (D > 0 && sizeof(TW) == 4 && !HD) {
+            const long long cols = (long long)P.n1 * (D == 1 ? P.n3 : P.n2);
+            const int nf = (D == 1 ? P.n2 : P.n3) + 1, L = march_length(cols, nf);
+            k_flux_march<D><<<dim3(cdiv(cols, 128), cdiv(nf, L)), 128, 0, s>>>(P, w, F, L);
+        } else {
+            constexpr int BX = FluxShape<D, TW, HD>::BX, BY = FluxShape<D, TW, HD>::BY;
+            int nx, ny, nz;
+            flux_tiles<D, BX, BY>(P, nx, ny, nz);
+            k_flux<D, TW, HD><<<dim3(nx, ny, nz), dim3(BX, BY), 0, s>>>(P, w, F);
+        }
     }
     static void flux_dir(const Params &P, int dir, const void *W, void *F, cudaStream_t s)
     {
