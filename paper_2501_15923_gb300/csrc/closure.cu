@@ -658,20 +658,26 @@ __global__ void __launch_bounds__(256, 1) k_conv_wgrad_tc(const __grid_constant_
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "n"(TCOLS) : "memory");
 }
 
-// dw[o][t][c] += the blocks' partial sums of row (d1 + 1) O + o, column line C + c, t = 3 line + d1 + 1
+// dw[o][t][c] += the blocks' partial sums of row (d1 + 1) O + o, column line C + c, t = 3 line + d1 + 1. A block
+// takes 32 neighbouring outputs, a warp every eighth partial of them (bound by the latency of the loads)
 template <int C, int O>
-__global__ void k_wgrad_reduce(const float *__restrict__ part, int nblk, float *dw)
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float *__restrict__ part, int nblk, float *dw)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= O * 27 * C) return;
+    __shared__ float ss[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;   // O 27 C is a multiple of 32
     const int c = e % C, t = (e / C) % 27, o = e / (27 * C);
-    const int row = (t % 3) * O + o, col = (t / 3) * C + c;
+    const float *p = part + ((long long)((t % 3) * O + o)) * (9 * C) + (t / 3) * C + c;
     float s = 0.f;
-#pragma unroll 16
-    for (int b = 0; b < nblk; ++b) s += part[((long long)b * 3 * O + row) * (9 * C) + col];
-    dw[e] += s;
+#pragma unroll 8
+    for (int b = w; b < nblk; b += 8) s += p[(long long)b * 3 * O * (9 * C)];
+    ss[w][lane] = s;
+    __syncthreads();
+    if (w == 0) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q) s += ss[q][lane];
+        dw[e] += s;
+    }
 }
-
 
 // ---- normalisation, loss, correction, optimiser --------------------------------------------------
 // x[z][c] = (U[c][v] - mean[c][i]) / scale[c][i] for c < 8, 0 for c in [8, 16)
@@ -760,18 +766,38 @@ __global__ void k_unpack_dU(Geo g, const float *__restrict__ y, const double *__
     for (int f = 0; f < NV; ++f) dU[f * g.N + v] = widen_f2d(y[(long long)v * 16 + f]) * oscale[f * g.n1 + i];
 }
 
-// Adam (FP32 master weights) and refresh of the BF16 copies w[O][27][C] and wt[C][27][O]
-__global__ void k_adam(int n, float *w, float *m, float *v, const float *grad, float lr, float b1, float b2, float eps,
-                       float c1, float c2)
+// one layer's weights, their moments, gradients and BF16 copies w[O][27][C] and wt[C][27][O]
+struct AdamLayer {
+    float *w, *mw, *vw, *dw, *b, *mb, *vb, *db;
+    bf16 *wb, *wt;
+    int O, C;
+};
+struct AdamLayers { AdamLayer l[4]; };
+
+__device__ __forceinline__ void adam_one(float *w, float *m, float *v, const float *grad, int q, float lr, float b1, float b2,
+                                         float eps, float c1, float c2)
 {
-    int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
     float gq = grad[q];
     float mq = b1 * m[q] + (1.f - b1) * gq;
     float vq = b2 * v[q] + (1.f - b2) * gq * gq;
     m[q] = mq;
     v[q] = vq;
     w[q] -= lr * (mq / c1) / (sqrtf(vq / c2) + eps);
+}
+
+// Adam (FP32 master weights) and the BF16 copies of all four layers in one launch (blockIdx.y: the layer;
+// its last threads take the biases): eight Adam and four copy launches of 3-4 us each before
+__global__ void k_adam(AdamLayers a, float lr, float b1, float b2, float eps, float c1, float c2)
+{
+    const AdamLayer &L = a.l[blockIdx.y];
+    const int n = L.O * 27 * L.C, q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < n) {
+        adam_one(L.w, L.mw, L.vw, L.dw, q, lr, b1, b2, eps, c1, c2);
+        const int c = q % L.C, t = (q / L.C) % 27, o = q / (27 * L.C);
+        const bf16 x = __float2bfloat16_rn(L.w[q]);
+        L.wb[q] = x;
+        L.wt[((long long)c * 27 + (26 - t)) * L.O + o] = x;      // transposed, taps reversed
+    } else if (q < n + L.O) adam_one(L.b, L.mb, L.vb, L.db, q - n, lr, b1, b2, eps, c1, c2);
 }
 
 __global__ void k_weights_bf16(int O, int C, const float *w, bf16 *wb, bf16 *wt)
@@ -965,7 +991,7 @@ void launch_wgrad_tc(Geo g, const bf16 *dpre, const bf16 *in, float *dw, float *
         return;
     }
     k_conv_wgrad_tc<C, O><<<nb, 256, wg_smem_bytes<C, O>(), s>>>(ta, tb, g, part, p_lo, p_hi, chunk);
-    k_wgrad_reduce<C, O><<<ccdiv(O * 27 * C, 256), 256, 0, s>>>(part, nb, dw);
+    k_wgrad_reduce<C, O><<<O * 27 * C / 32, 256, 0, s>>>(part, nb, dw);
 }
 
 // floats of the partial-sum buffer of launch_wgrad (one block per SM, 3 x 32 rows x 9 x 32 columns)
@@ -1013,6 +1039,8 @@ struct icarus_closure {
     float *wpart;          // partial sums of the weight-gradient blocks
     float *y, *dy;         // [N][16]
     double *mean, *scale, *oscale, *loss, *upack;
+    float *grads = nullptr;   // [loss (2 floats) | dw, db of each layer]
+    size_t n_grads = 0;
     int step = 0;
     bool have_norm = false;
 };
@@ -1096,6 +1124,12 @@ int icarus_closure_create(int n1, int n2, int n3, unsigned long long seed, void 
     const Geo &g = c->g;
     bool ok = true;
     uint64_t st = seed;
+    // the gradients of all layers and the loss (first, 8 bytes) in one block, cleared together
+    size_t ng = 2, goff = 2;
+    for (int l = 0; l < 4; ++l) ng += LO[l] * 27 * LC[l] + LO[l];
+    c->n_grads = ng;
+    c->grads = (float *)cl_alloc(c, ng * 4);
+    c->loss = (double *)c->grads;
     for (int l = 0; l < 4; ++l) {
         const int n = LO[l] * 27 * LC[l];
         std::vector<float> hw(n, 0.f), hb(LO[l], 0.f);
@@ -1104,9 +1138,10 @@ int icarus_closure_create(int n1, int n2, int n3, unsigned long long seed, void 
             for (int t = 0; t < 27; ++t)
                 for (int ci = 0; ci < RC[l]; ++ci) hw[((size_t)o * 27 + t) * LC[l] + ci] = (float)(sd * gauss(st));
         c->w[l] = (float *)cl_alloc(c, n * 4); c->mw[l] = (float *)cl_alloc(c, n * 4);
-        c->vw[l] = (float *)cl_alloc(c, n * 4); c->dw[l] = (float *)cl_alloc(c, n * 4);
+        c->vw[l] = (float *)cl_alloc(c, n * 4); c->dw[l] = c->grads ? c->grads + goff : nullptr;
         c->b[l] = (float *)cl_alloc(c, LO[l] * 4); c->mb[l] = (float *)cl_alloc(c, LO[l] * 4);
-        c->vb[l] = (float *)cl_alloc(c, LO[l] * 4); c->db[l] = (float *)cl_alloc(c, LO[l] * 4);
+        c->vb[l] = (float *)cl_alloc(c, LO[l] * 4); c->db[l] = c->grads ? c->grads + goff + n : nullptr;
+        goff += n + LO[l];
         c->wb[l] = (bf16 *)cl_alloc(c, n * 2); c->wt[l] = (bf16 *)cl_alloc(c, n * 2);
         if (!c->w[l] || !c->mw[l] || !c->vw[l] || !c->dw[l] || !c->b[l] || !c->mb[l] || !c->vb[l] || !c->db[l] ||
             !c->wb[l] || !c->wt[l]) { ok = false; break; }
@@ -1128,7 +1163,6 @@ int icarus_closure_create(int n1, int n2, int n3, unsigned long long seed, void 
         c->mean = (double *)cl_alloc(c, 8 * n1 * 8);
         c->scale = (double *)cl_alloc(c, 8 * n1 * 8);
         c->oscale = (double *)cl_alloc(c, 8 * n1 * 8);
-        c->loss = (double *)cl_alloc(c, 8);
         c->upack = (double *)cl_alloc(c, 8 * g.N * 8);
         c->wpart = (float *)cl_alloc(c, wgrad_part_floats() * 4);
         ok = c->dpre && c->din && c->y && c->dy && c->mean && c->scale && c->oscale && c->loss && c->upack && c->wpart;
@@ -1176,12 +1210,8 @@ int icarus_closure_train_step(icarus_closure *c, const double *U_in, const doubl
     k_pad_fill<bf16><<<ccdiv(g.NP, 256), 256, 0, s>>>(g, c->act[0], 16);
     forward(c);
     if (tc_map_failed()) return report_error(ICARUS_ECUDA, "tensor map encoding failed");
-    CCK(cudaMemsetAsync(c->loss, 0, 8, s));
+    CCK(cudaMemsetAsync(c->grads, 0, c->n_grads * 4, s));
     k_mse<<<ccdiv(g.N, 256), 256, 0, s>>>(g, c->y, dU_target, c->oscale, c->dy, c->loss);
-    for (int l = 0; l < 4; ++l) {
-        CCK(cudaMemsetAsync(c->dw[l], 0, LO[l] * 27 * LC[l] * 4, s));
-        CCK(cudaMemsetAsync(c->db[l], 0, LO[l] * 4, s));
-    }
     // layer 3 (linear): gradient from the loss; then ReLU layers with the mask of their output
     for (int l = 3; l >= 0; --l) {
         if (l == 3) launch_dpre(LO[l], g, c->dy, 0, nullptr, c->dpre, c->db[l], s);
@@ -1195,13 +1225,11 @@ int icarus_closure_train_step(icarus_closure *c, const double *U_in, const doubl
     c->step++;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - powf(b1, (float)c->step), c2 = 1.f - powf(b2, (float)c->step);
-    for (int l = 0; l < 4; ++l) {
-        int n = LO[l] * 27 * LC[l];
-        k_adam<<<ccdiv(n, 256), 256, 0, s>>>(n, c->w[l], c->mw[l], c->vw[l], c->dw[l], (float)lr, b1, b2, 1e-8f, c1, c2);
-        k_adam<<<1, 64, 0, s>>>(LO[l], c->b[l], c->mb[l], c->vb[l], c->db[l], (float)lr, b1, b2, 1e-8f, c1, c2);
-    }
-    int rc = refresh_bf16(c);
-    if (rc) return rc;
+    AdamLayers al;
+    for (int l = 0; l < 4; ++l)
+        al.l[l] = AdamLayer{c->w[l], c->mw[l], c->vw[l], c->dw[l], c->b[l], c->mb[l], c->vb[l], c->db[l], c->wb[l], c->wt[l], LO[l], LC[l]};
+    k_adam<<<dim3(ccdiv(32 * 27 * 32 + 32, 256), 4), 256, 0, s>>>(al, (float)lr, b1, b2, 1e-8f, c1, c2);
+    CCK(cudaGetLastError());
     if (loss) {
         CCK(cudaMemcpyAsync(loss, c->loss, 8, cudaMemcpyDeviceToHost, s));
         CCK(cudaStreamSynchronize(s));
