@@ -114,7 +114,8 @@ void dfree_all(icarus_ctx *c)
 void drop_graph(icarus_ctx *c)
 {
     if (c->graph) cudaGraphExecDestroy(c->graph);
-    c->graph = nullptr;
+    if (c->graph_k) cudaGraphExecDestroy(c->graph_k);
+    c->graph = c->graph_k = nullptr;
     c->p_version++;
 }
 
@@ -299,15 +300,17 @@ bool use_update_rf(const icarus_ctx *c)
            c->opts.divb != ICARUS_DIVB_GLM && !c->opts.tracer;
 }
 
-void enqueue_step(icarus_ctx *c, cudaStream_t s)
+// one step up to its probes; the second stage's update, the first kernel to change what the previous
+// step's probes read (the interior primitives, the time), waits for `probed` when given
+void enqueue_stages(icarus_ctx *c, cudaStream_t s, cudaEvent_t probed)
 {
     const Params &P = c->P;
     if (use_fused_stage(c)) {
         c->ops.fill_ghosts(P, c->W, 1, s);
         c->ops.fused_stage(P, 1, c->U, c->W, c->U1, c->W1, s);
         c->ops.fill_ghosts(P, c->W1, 2, s);
+        if (probed) cudaStreamWaitEvent(s, probed, 0);
         c->ops.fused_stage(P, 2, c->U1, c->W1, c->U, c->W, s);
-        if (P.n_probes > 0) c->ops.probe(P, c->W, s);
         return;
     }
     // stage 1: U, W at t  ->  U1, W1 (tracer: rho c in T, c in C  ->  T1, C1, with the stage's mass fluxes)
@@ -332,11 +335,17 @@ void enqueue_step(icarus_ctx *c, cudaStream_t s)
     else if (rf) { c->ops.flux_dir(P, 1, c->W1, c->F2, s); c->ops.flux_dir(P, 2, c->W1, c->F3, s); }
     else c->ops.fluxes(P, c->W1, c->F1, c->F2, c->F3, s);
     if (P.divb == 1 || P.divb == 3) c->ops.divb(P, c->W1, c->divB, s);
+    if (probed) cudaStreamWaitEvent(s, probed, 0);
     if (rf) c->ops.update_rf(P, 2, c->U1, c->W1, c->U, c->W, c->F2, c->F3, c->divB, s);
     else c->ops.update(P, 2, c->U1, c->W1, c->U, c->W, c->F1, c->F2, c->F3, c->divB, s);
     if (glm) c->ops.glm_update(P, 2, c->Psi1, c->Psi, c->FP1, c->FP2, c->FP3, s);
     if (tr) c->ops.tracer_update(P, 2, c->C1, c->F1, c->F2, c->F3, c->T1, c->T, c->U, c->C, s);
-    if (P.n_probes > 0) c->ops.probe(P, c->W, s);
+}
+
+void enqueue_step(icarus_ctx *c, cudaStream_t s)
+{
+    enqueue_stages(c, s, nullptr);
+    if (c->P.n_probes > 0) c->ops.probe(c->P, c->W, s);
 }
 
 int count_launches(const icarus_ctx *c)
@@ -360,6 +369,43 @@ int build_graph(icarus_ctx *c)
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return fail(ICARUS_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
     c->launches_per_step = count_launches(c);
+    return ICARUS_OK;
+}
+
+// STEPS_K steps in one graph: one launch instead of STEPS_K (no gap between the steps), and each step's probe
+// kernel, one block bound by latency, runs on a branch beside the next step's kernels up to its second
+// update. 20 steps with probes at 60 x 16 x 32: 183 -> 175 us a step, 300 x 33 x 65 FP32: 194 -> 185
+constexpr int STEPS_K = 4;
+
+int build_graph_k(icarus_ctx *c)
+{
+    const bool probes = c->P.n_probes > 0;
+    if (probes && !c->side) {
+        CK(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+        CK(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
+        CK(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+    }
+    cudaGraph_t g;
+    CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
+    cudaError_t e = cudaSuccess;
+    auto ok = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
+    for (int q = 0; q < STEPS_K; ++q) {
+        enqueue_stages(c, c->stream, probes && q > 0 ? c->ev_join : nullptr);
+        if (!probes) continue;
+        ok(cudaEventRecord(c->ev_fork, c->stream));
+        ok(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+        c->ops.probe(c->P, c->W, c->side);
+        ok(cudaEventRecord(c->ev_join, c->side));
+    }
+    if (probes) ok(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
+    const cudaError_t e2 = cudaStreamEndCapture(c->stream, &g);
+    if (e == cudaSuccess && e2 == cudaSuccess) {
+        e = cudaGraphInstantiate(&c->graph_k, g, 0);
+        if (e != cudaSuccess) c->graph_k = nullptr;
+    }
+    if (e2 == cudaSuccess) cudaGraphDestroy(g);
+    if (e != cudaSuccess || e2 != cudaSuccess)
+        return fail(ICARUS_ECUDA, "graph capture: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
     return ICARUS_OK;
 }
 
@@ -656,6 +702,11 @@ int icarus_step(icarus_ctx *c, int n)
         int rc = build_graph(c);
         if (rc) return rc;
     }
+    if (n >= STEPS_K && !c->graph_k) {
+        int rc = build_graph_k(c);
+        if (rc) return rc;
+    }
+    for (; n >= STEPS_K; n -= STEPS_K) CK(cudaGraphLaunch(c->graph_k, c->stream));
     for (int q = 0; q < n; ++q) CK(cudaGraphLaunch(c->graph, c->stream));
     return ICARUS_OK;
 }
@@ -805,6 +856,9 @@ int icarus_destroy(icarus_ctx *c)
     dfree_all(c);
     if (c->hstage) cudaFreeHost(c->hstage);
     if (c->hstatus) cudaFreeHost(c->hstatus);
+    if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+    if (c->ev_join) cudaEventDestroy(c->ev_join);
+    if (c->side) cudaStreamDestroy(c->side);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
     return ICARUS_OK;

@@ -30,7 +30,10 @@ struct icarus_ctx {
     void *snapU = nullptr, *snapT = nullptr, *snapC = nullptr, *snapPsi = nullptr;   // icarus_step_recover's snapshot
     size_t hstage_cap = 0;
     bool have_state = false, have_boundary = false;
-    cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph = nullptr;       // one step
+    cudaGraphExec_t graph_k = nullptr;     // several steps, each step's probes beside the next step
+    cudaStream_t side = nullptr;           // (captured only) the probes' branch and its fork and join
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     long long ring_tail = 0;
     double t0, p0, b0, omega_code, gm_code;
     int launches_per_step = 0;
