@@ -481,11 +481,36 @@ __device__ __forceinline__ double vanleer_half(double a, double b, double s)
     return fma(fma(-q, s, p), r, q);
 }
 
-// half the limited slope in double precision (van Leer: one integer-pipe sum and vanleer_half)
+// half the limited slope in double precision, off the FP64 pipe but for vanleer_half's three operations:
+// van Leer a b / (a + b); minmod min(|a|, |b|) / 2; monotonised central min(|a|, |b|, |a + b| / 4), with
+// magnitudes compared as integers and the exact halvings on the exponent (as FP64 arithmetic these
+// took about ten operations a field)
+static __device__ __noinline__ double quarter_slow(double x) { return 0.25 * x; }
 __device__ __forceinline__ double half_slope(int lim, double a, double b)
 {
-    if (lim != 1) return half_r(limiter<double>(lim, a, b));
-    return (hi_bits(a) ^ hi_bits(b)) >= 0 && !is_zero(a) && !is_zero(b) ? vanleer_half(a, b, add_i(a, b)) : 0.0;
+    if ((hi_bits(a) ^ hi_bits(b)) < 0 || is_zero(a) || is_zero(b)) return 0.0;
+    if (lim == 1) return vanleer_half(a, b, add_i(a, b));
+    unsigned int ah, al, bh, bl;
+    split_d(a, ah, al);
+    split_d(b, bh, bl);
+    const unsigned long long ma = (unsigned long long)(ah & 0x7fffffffu) << 32 | al,
+                             mb = (unsigned long long)(bh & 0x7fffffffu) << 32 | bl;
+    unsigned long long m = ma < mb ? ma : mb;
+    const unsigned int sign = ah & 0x80000000u;
+    if (lim == 0) return half_r(join_d((unsigned int)(m >> 32) | sign, (unsigned int)m));
+    double t = add_i(a, b);
+    unsigned int th, tl;
+    split_d(t, th, tl);
+    const unsigned int e = (th >> 20) & 0x7ffu;
+    if (e == 0x7ffu) return t;                                   // NaN, or beyond the range
+    if (e >= 3u) th -= 2u << 20;
+    else {
+        t = quarter_slow(t);
+        split_d(t, th, tl);
+    }
+    const unsigned long long mt = (unsigned long long)(th & 0x7fffffffu) << 32 | tl;
+    m = mt < m ? mt : m;
+    return join_d((unsigned int)(m >> 32) | sign, (unsigned int)m);
 }
 
 // half the limited slope in single precision. van Leer 2 a b / (a + b) as the product with the hardware
@@ -686,6 +711,67 @@ __device__ __forceinline__ void tvdlf_d(const double *wl, const double *wr, int 
     f[4 + t2] = fma(-wl[t2], bl, fma(-wr[t2], br, f[4 + t2]));
 }
 
+// a < b for doubles that are not NaN, on the integer pipe (ordered like the sign-magnitude bit patterns)
+__device__ __forceinline__ bool less_i(double a, double b)
+{
+    unsigned int ah, al, bh, bl;
+    split_d(a, ah, al);
+    split_d(b, bh, bl);
+    const long long x = (long long)((unsigned long long)ah << 32 | al), y = (long long)((unsigned long long)bh << 32 | bl);
+    return (x < 0 ? (long long)0x8000000000000000ull - x : x) < (y < 0 ? (long long)0x8000000000000000ull - y : y);
+}
+
+// conserved state u and physical flux F along d of the primitives w
+__device__ __forceinline__ void state_flux_d(const double *w, int d, double igm1, double *u, double *F)
+{
+    const int n = 1 + d;
+    const double vn = w[n], bn = w[4 + n];
+    u[RHO] = w[0];
+    u[M1] = w[0] * w[1];
+    u[M2] = w[0] * w[2];
+    u[M3] = w[0] * w[3];
+    const double bb = fma(w[5], w[5], fma(w[6], w[6], w[7] * w[7]));
+    const double bv = fma(w[5], w[1], fma(w[6], w[2], w[7] * w[3])), pt = fma(0.5, bb, w[4]);
+    u[EN] = fma(w[4], igm1, half_r(fma(u[M1], w[1], fma(u[M2], w[2], u[M3] * w[3])) + bb));
+    u[B1] = w[5]; u[B2] = w[6]; u[B3] = w[7];
+    F[RHO] = u[n];
+#pragma unroll
+    for (int c = 1; c < 4; ++c) {
+        F[c] = fma(u[c], vn, c == n ? fma(-bn, bn, pt) : -(w[4 + c] * bn));
+        F[4 + c] = c == n ? 0.0 : fma(vn, w[4 + c], -(bn * w[c]));   // the normal component is exactly zero
+    }
+    F[EN] = fma(u[EN] + pt, vn, -(bn * bv));
+}
+
+// double-precision HLL: the signal speeds first, then only the side(s) the face needs (one where it is
+// supersonic, as most r faces of the wind are); between them the combination with weights formed once,
+// S_R F_L / D - S_L F_R / D + S_L S_R (U_R - U_L) / D, three FP64 operations a field instead of five
+__device__ __forceinline__ void hll_d(const double *wl, const double *wr, int d, double gamma, double igm1, double irl, double irr,
+                                      double *f)
+{
+    const int n = 1 + d;
+    double c[2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const double *w = s ? wr : wl;
+        const double bb = fma(w[5], w[5], fma(w[6], w[6], w[7] * w[7])), a = gamma * w[4], S = a + bb, bn = w[4 + n];
+        const double disc = clamp0_r(fma(S, S, -(quad_r(a) * (bn * bn))));
+        c[s] = sqrt_nr(half_r(S + sqrt_nr(disc)) * (s ? irr : irl));
+    }
+    const double l0 = sub_i(wl[n], c[0]), l1 = sub_i(wr[n], c[1]), r0 = add_i(wl[n], c[0]), r1 = add_i(wr[n], c[1]);
+    const double sl = less_i(l0, l1) ? l0 : l1, sr = less_i(r0, r1) ? r1 : r0;
+    double u[NV];
+    if (!less_i(sl, 0.0)) { state_flux_d(wl, d, igm1, u, f); return; }
+    if (!less_i(0.0, sr)) { state_flux_d(wr, d, igm1, u, f); return; }
+    double ur[NV], fr[NV];
+    state_flux_d(wl, d, igm1, u, f);
+    state_flux_d(wr, d, igm1, ur, fr);
+    const double q = rcp_nr(sr - sl), a = sr * q, b = sl * q, e = a * sl;
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+        f[v] = v == 4 + n ? e * sub_i(ur[v], u[v]) : fma(a, f[v], fma(-b, fr[v], e * sub_i(ur[v], u[v])));
+}
+
 // TVDLF: (F_L + F_R)/2 - c_max (U_R - U_L)/2; HLL with signal speeds from the fast speeds (flux
 // chosen at run time); HLLD when HD (a separate instantiation, so that the larger solver does not
 // weigh on the registers of the other two)
@@ -721,10 +807,9 @@ __device__ __forceinline__ void riemann(const R *wl, const R *wr, int d, int flu
         irr = R(1) / wr[0];
     }
     if constexpr (sizeof(R) == 8 && !HD) {
-        if (flux == 0) {
-            tvdlf_d(wl, wr, d, gamma, igm1, irl, irr, f);
-            return;
-        }
+        if (flux == 0) tvdlf_d(wl, wr, d, gamma, igm1, irl, irr, f);
+        else hll_d(wl, wr, d, gamma, igm1, irl, irr, f);
+        return;
     }
     R ul[NV], ur[NV];
     prim2cons(wl, ul, igm1);
