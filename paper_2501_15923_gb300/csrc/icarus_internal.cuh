@@ -223,8 +223,7 @@ __device__ __forceinline__ double join_d(unsigned int hi, unsigned int lo)
 // x + y, or x - y with flip = 0x80000000, on the integer pipe, to the bit what the FP64 pipe gives (round
 // to nearest even): the larger magnitude's mantissa with ten guard bits, the other shifted to it with
 // its lost bits jammed into the last, summed in two's complement, normalised and rounded. Sums
-// outside the normal range, of infinities or NaN, or cancelling by more than 2^30 but not to zero take
-// the FP64 addition. About 65 instructions, 32 of the integer pipe's cycles for a warp, beside an FP64
+// outside the normal range, of infinities or NaN take the FP64 addition. About 65 instructions, 32 of the integer pipe's cycles for a warp, beside an FP64
 // instruction's 19 of the FP64 pipe's: worth it where the FP64 pipe is the bound and the others idle.
 // (a call: a branch this short would become a predicated FP64 instruction, which takes its turn on the
 // FP64 pipe with every lane off)
@@ -253,10 +252,11 @@ struct AddI {
     __device__ __forceinline__ double sum(int t, unsigned int hs, unsigned int hz, double x, double y, bool minus) const
     {
         unsigned long long S = ma + ((ms ^ (unsigned long long)(long long)t) + (unsigned long long)(t & 1));
-        const unsigned int sh = (unsigned int)(S >> 32);
-        if (__builtin_expect(S != 0ull && (sh == 0u || (unsigned int)(ea - 64) > 1900u), 0)) return add_slow(x, y, minus);
-        const int n = __clz((int)sh);
-        S <<= n;
+        if (__builtin_expect(S != 0ull && (unsigned int)(ea - 64) > 1900u, 0)) return add_slow(x, y, minus);
+        const bool low = (unsigned int)(S >> 32) == 0u;           // cancelled by 2^30 or more (exact)
+        if (low) S <<= 32;
+        const int n0 = __clz((int)(unsigned int)(S >> 32)), n = low ? n0 + 32 : n0;
+        S <<= n0;
         const unsigned long long m = S >> 11;
         const unsigned int up = ((unsigned int)S & 0x7ffu) + ((unsigned int)m & 1u) > 0x400u ? 1u : 0u;
         const unsigned long long r = m + up + ((unsigned long long)((unsigned int)(ea - n) << 20 | (hs & 0x80000000u)) << 32);
