@@ -380,7 +380,7 @@ __device__ __forceinline__ void flux_tile(const Params &P, const TW *__restrict_
 // The FP64 flux tile (TVDLF / HLL). The FP64 pipe bounds it (a warp's instruction takes 19 cycles of an
 // SM's pipe; the other pipes idled), so what can run elsewhere does: the differences, slope sums and
 // face values are additions on the integer pipe (add_i, to the bit the FP64 result), which leaves
-// three FP64 operations a field, 115 a face instead of 155. The reconstruction is a loop over the
+// three FP64 operations a field, 93-102 a face instead of 155. The reconstruction is a loop over the
 // fields, one field's stencil in registers at a time, both face states through shared memory:
 // unrolled over the eight fields the integer code does not fit the instruction cache (r flux 1.35 ms
 // against 1.03 for the same additions). r / theta / phi flux at 512 x 64 x 128: 1.30 / 1.33 / 1.27 ->
