@@ -250,6 +250,13 @@ int icarus_time(icarus_ctx *ctx, double *t, double *dt);
  * 1 / x[i]. Synchronous; a temporary device buffer. EINVAL for n outside [1, 2^24] or NULL. */
 int icarus_math_check(int n, const double *x, double *y);
 
+/* The same check of the additions that the FP64 flux kernels form on the integer pipe (to the bit what
+ * the FP64 pipe gives, infinities and NaN included) and of their half limited slopes: for the n pairs of
+ * host values (a, b), y[5i .. 5i + 4] receive a + b, a - b, both again from the form that shares their
+ * alignment, and half the slope of the differences a and b under `limiter`. Synchronous; a temporary
+ * device buffer. EINVAL for n outside [1, 2^24], an unknown limiter or NULL. */
+int icarus_pair_check(int n, int limiter, const double *a, const double *b, double *y);
+
 /* Measured fused multiply-add rate of the current GPU (not part of the paper's method; the
  * denominator of the arithmetic roofline of the FP64 kernels, whose bound is the FP64 pipe):
  * blocks_per_sm x SMs blocks of 256 threads, each thread `chains` (1, 4, 8 or 16) independent

@@ -98,6 +98,21 @@ __global__ void k_math_check(const double *x, double *y, int n)
     }
 }
 
+// the FP64 flux kernels' integer additions and half slope of pairs (a, b): y[5i .. 5i + 4] = add_i, sub_i,
+// the sum and the difference of add_sub_i, half_slope
+__global__ void k_pair_check(const double *a, const double *b, double *y, int limiter, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double s, d;
+    add_sub_i(a[i], b[i], s, d);
+    y[5LL * i] = add_i(a[i], b[i]);
+    y[5LL * i + 1] = sub_i(a[i], b[i]);
+    y[5LL * i + 2] = s;
+    y[5LL * i + 3] = d;
+    y[5LL * i + 4] = half_slope(limiter, a[i], b[i]);
+}
+
 }  // namespace
 
 namespace {
@@ -1004,6 +1019,25 @@ int icarus_math_check(int n, const double *x, double *y)
     if (e == cudaSuccess) e = cudaMemcpy(y, d + n, (size_t)4 * n * sizeof(double), cudaMemcpyDeviceToHost);
     cudaFree(d);
     if (e != cudaSuccess) return fail(ICARUS_ECUDA, "math check: %s", cudaGetErrorString(e));
+    return ICARUS_OK;
+}
+
+int icarus_pair_check(int n, int limiter, const double *a, const double *b, double *y)
+{
+    if (n < 1 || n > (1 << 24) || !a || !b || !y) return fail(ICARUS_EINVAL, "n in [1, 2^24], a, b and y host arrays");
+    if (limiter < 0 || limiter > 2) return fail(ICARUS_EINVAL, "bad limiter");
+    double *d = nullptr;
+    const size_t sz = (size_t)n * sizeof(double);
+    CK(cudaMalloc(&d, 7 * sz));
+    cudaError_t e = cudaMemcpy(d, a, sz, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d + n, b, sz, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        k_pair_check<<<(n + 255) / 256, 256>>>(d, d + n, d + 2LL * n, limiter, n);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(y, d + 2LL * n, 5 * sz, cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    if (e != cudaSuccess) return fail(ICARUS_ECUDA, "pair check: %s", cudaGetErrorString(e));
     return ICARUS_OK;
 }
 

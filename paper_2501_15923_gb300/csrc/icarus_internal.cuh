@@ -220,11 +220,12 @@ __device__ __forceinline__ double join_d(unsigned int hi, unsigned int lo)
     return x;
 }
 
-// x + y, or x - y with flip = 0x80000000, on the integer pipe, to the bit what the FP64 pipe gives (round
-// to nearest even): the larger magnitude's mantissa with ten guard bits, the other shifted to it with
-// its lost bits jammed into the last, summed in two's complement, normalised and rounded. Sums
-// outside the normal range, of infinities or NaN take the FP64 addition. About 65 instructions, 32 of the integer pipe's cycles for a warp, beside an FP64
-// instruction's 19 of the FP64 pipe's: worth it where the FP64 pipe is the bound and the others idle.
+// x + y and x - y on the integer pipe, to the bit what the FP64 pipe gives (round to nearest even): the
+// larger magnitude's mantissa with ten guard bits, the other shifted to it with its lost bits jammed
+// into the last, summed in two's complement, normalised and rounded. Sums that could leave the normal
+// range and those of infinities or NaN take the FP64 addition. About 65 instructions, 32 of the integer
+// pipe's cycles for a warp, beside an FP64 instruction's 19 of the FP64 pipe's: worth it where the FP64
+// pipe is the bound and the others idle.
 // (a call: a branch this short would become a predicated FP64 instruction, which takes its turn on the
 // FP64 pipe with every lane off)
 static __device__ __noinline__ double add_slow(double x, double y, bool minus) { return minus ? x - y : x + y; }
@@ -252,7 +253,9 @@ struct AddI {
     __device__ __forceinline__ double sum(int t, unsigned int hs, unsigned int hz, double x, double y, bool minus) const
     {
         unsigned long long S = ma + ((ms ^ (unsigned long long)(long long)t) + (unsigned long long)(t & 1));
-        if (__builtin_expect(S != 0ull && (unsigned int)(ea - 64) > 1900u, 0)) return add_slow(x, y, minus);
+        // (zeros, which whole fields may hold, stay here: S | ea is zero for them only)
+        if (__builtin_expect((unsigned int)(ea - 64) > 1900u && ((unsigned int)S | (unsigned int)(S >> 32) | (unsigned int)ea) != 0u, 0))
+            return add_slow(x, y, minus);
         const bool low = (unsigned int)(S >> 32) == 0u;           // cancelled by 2^30 or more (exact)
         if (low) S <<= 32;
         const int n0 = __clz((int)(unsigned int)(S >> 32)), n = low ? n0 + 32 : n0;

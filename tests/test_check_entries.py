@@ -1,0 +1,22 @@
+"""Argument checks of the entry points that expose the kernels' own arithmetic (rejected before any CUDA
+call, so no GPU is needed)."""
+import ctypes as C
+
+import pytest
+
+EINVAL = -1
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_2501_15923_gb300 import build
+    build.build()
+    from paper_2501_15923_gb300 import icarus
+    return icarus.load()
+
+
+def test_pair_check(lib):
+    x, y = (C.c_double * 2)(1.0, 2.0), (C.c_double * 10)()
+    for args in ((0, 1, x, x, y), ((1 << 24) + 1, 1, x, x, y), (2, 3, x, x, y), (2, -1, x, x, y), (2, 1, None, x, y),
+                 (2, 1, x, None, y), (2, 1, x, x, None)):
+        assert lib.icarus_pair_check(*args) == EINVAL, args
