@@ -257,6 +257,12 @@ int icarus_math_check(int n, const double *x, double *y);
  * device buffer. EINVAL for n outside [1, 2^24], an unknown limiter or NULL. */
 int icarus_pair_check(int n, int limiter, const double *a, const double *b, double *y);
 
+/* The FP64 TVDLF or HLL flux across faces normal to direction dir (0, 1, 2), as the flux kernels form it:
+ * host arrays of left and right states wl, wr [n][8] (rho, v, p, B in code units) to f [n][8] (fluxes of
+ * rho, rho v, e, B). Synchronous; a temporary device buffer. EINVAL for n outside [1, 2^22], another
+ * direction or flux, gamma <= 1 or NULL. */
+int icarus_face_check(int n, int dir, int flux, double gamma, const double *wl, const double *wr, double *f);
+
 /* Measured fused multiply-add rate of the current GPU (not part of the paper's method; the
  * denominator of the arithmetic roofline of the FP64 kernels, whose bound is the FP64 pipe):
  * blocks_per_sm x SMs blocks of 256 threads, each thread `chains` (1, 4, 8 or 16) independent

@@ -113,6 +113,22 @@ __global__ void k_pair_check(const double *a, const double *b, double *y, int li
     y[5LL * i + 4] = half_slope(limiter, a[i], b[i]);
 }
 
+// the FP64 TVDLF / HLL flux along dir of face states wl, wr [n][8]
+__global__ void k_face_check(const double *wl, const double *wr, double *f, int dir, int flux, double gamma, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double l[NV], r[NV], y[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) { l[v] = wl[8LL * i + v]; r[v] = wr[8LL * i + v]; }
+    const double igm1 = 1.0 / (gamma - 1.0);
+    if (dir == 0) riemann<double>(l, r, 0, flux, gamma, igm1, y);
+    else if (dir == 1) riemann<double>(l, r, 1, flux, gamma, igm1, y);
+    else riemann<double>(l, r, 2, flux, gamma, igm1, y);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) f[8LL * i + v] = y[v];
+}
+
 }  // namespace
 
 namespace {
@@ -1038,6 +1054,26 @@ int icarus_pair_check(int n, int limiter, const double *a, const double *b, doub
     if (e == cudaSuccess) e = cudaMemcpy(y, d + 2LL * n, 5 * sz, cudaMemcpyDeviceToHost);
     cudaFree(d);
     if (e != cudaSuccess) return fail(ICARUS_ECUDA, "pair check: %s", cudaGetErrorString(e));
+    return ICARUS_OK;
+}
+
+int icarus_face_check(int n, int dir, int flux, double gamma, const double *wl, const double *wr, double *f)
+{
+    if (n < 1 || n > (1 << 22) || !wl || !wr || !f) return fail(ICARUS_EINVAL, "n in [1, 2^22], wl, wr and f host arrays");
+    if (dir < 0 || dir > 2 || (flux != ICARUS_FLUX_TVDLF && flux != ICARUS_FLUX_HLL) || !(gamma > 1.0))
+        return fail(ICARUS_EINVAL, "bad direction, flux (TVDLF or HLL) or gamma");
+    double *d = nullptr;
+    const size_t sz = (size_t)8 * n * sizeof(double);
+    CK(cudaMalloc(&d, 3 * sz));
+    cudaError_t e = cudaMemcpy(d, wl, sz, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d + 8LL * n, wr, sz, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        k_face_check<<<(n + 127) / 128, 128>>>(d, d + 8LL * n, d + 16LL * n, dir, flux, gamma, n);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(f, d + 16LL * n, sz, cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    if (e != cudaSuccess) return fail(ICARUS_ECUDA, "face check: %s", cudaGetErrorString(e));
     return ICARUS_OK;
 }
 

@@ -714,14 +714,29 @@ __device__ __forceinline__ void tvdlf_d(const double *wl, const double *wr, int 
     f[4 + t2] = fma(-wl[t2], bl, fma(-wr[t2], br, f[4 + t2]));
 }
 
-// a < b for doubles that are not NaN, on the integer pipe (ordered like the sign-magnitude bit patterns)
+// a < b (-0 below +0), x >= 0 and x <= 0 on the integer pipe from the sign-magnitude bit patterns, false for
+// NaN: of results of an addition, whose NaN shows in the high word
 __device__ __forceinline__ bool less_i(double a, double b)
 {
     unsigned int ah, al, bh, bl;
     split_d(a, ah, al);
     split_d(b, bh, bl);
-    const long long x = (long long)((unsigned long long)ah << 32 | al), y = (long long)((unsigned long long)bh << 32 | bl);
-    return (x < 0 ? (long long)0x8000000000000000ull - x : x) < (y < 0 ? (long long)0x8000000000000000ull - y : y);
+    const unsigned int as = (unsigned int)((int)ah >> 31), bs = (unsigned int)((int)bh >> 31);
+    const long long x = (long long)((unsigned long long)(ah ^ (as >> 1)) << 32 | (al ^ as));
+    const long long y = (long long)((unsigned long long)(bh ^ (bs >> 1)) << 32 | (bl ^ bs));
+    return x < y && max(ah & 0x7fffffffu, bh & 0x7fffffffu) <= 0x7ff00000u;
+}
+__device__ __forceinline__ bool not_negative_i(double x)
+{
+    unsigned int h, l;
+    split_d(x, h, l);
+    return h <= 0x7ff00000u || (h << 1 | l) == 0u;
+}
+__device__ __forceinline__ bool not_positive_i(double x)
+{
+    unsigned int h, l;
+    split_d(x, h, l);
+    return h - 0x80000000u <= 0x7ff00000u || (h | l) == 0u;
 }
 
 // conserved state u and physical flux F along d of the primitives w
@@ -762,10 +777,10 @@ __device__ __forceinline__ void hll_d(const double *wl, const double *wr, int d,
         c[s] = sqrt_nr(half_r(S + sqrt_nr(disc)) * (s ? irr : irl));
     }
     const double l0 = sub_i(wl[n], c[0]), l1 = sub_i(wr[n], c[1]), r0 = add_i(wl[n], c[0]), r1 = add_i(wr[n], c[1]);
-    const double sl = less_i(l0, l1) ? l0 : l1, sr = less_i(r0, r1) ? r1 : r0;
+    const double sl = less_i(l0, l1) ? l0 : l1, sr = less_i(r1, r0) ? r0 : r1;
     double u[NV];
-    if (!less_i(sl, 0.0)) { state_flux_d(wl, d, igm1, u, f); return; }
-    if (!less_i(0.0, sr)) { state_flux_d(wr, d, igm1, u, f); return; }
+    if (not_negative_i(sl)) { state_flux_d(wl, d, igm1, u, f); return; }
+    if (not_positive_i(sr)) { state_flux_d(wr, d, igm1, u, f); return; }
     double ur[NV], fr[NV];
     state_flux_d(wl, d, igm1, u, f);
     state_flux_d(wr, d, igm1, ur, fr);

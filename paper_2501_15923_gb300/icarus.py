@@ -71,6 +71,7 @@ SIGNATURES = {
     "icarus_status": (C.c_int, [C.c_void_p, C.POINTER(C.c_longlong)]),
     "icarus_math_check": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p]),
     "icarus_pair_check": (C.c_int, [C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]),
+    "icarus_face_check": (C.c_int, [C.c_int, C.c_int, C.c_int, C.c_double, C.c_void_p, C.c_void_p, C.c_void_p]),
     "icarus_scales": (C.c_int, [C.c_void_p, C.c_void_p]),
     "icarus_launches_per_step": (C.c_int, [C.c_void_p]),
     "icarus_get_stream": (C.c_void_p, [C.c_void_p]),

@@ -20,3 +20,11 @@ def test_pair_check(lib):
     for args in ((0, 1, x, x, y), ((1 << 24) + 1, 1, x, x, y), (2, 3, x, x, y), (2, -1, x, x, y), (2, 1, None, x, y),
                  (2, 1, x, None, y), (2, 1, x, x, None)):
         assert lib.icarus_pair_check(*args) == EINVAL, args
+
+
+def test_face_check(lib):
+    w, f = (C.c_double * 16)(*([1.0] * 16)), (C.c_double * 16)()
+    for args in ((0, 0, 0, 1.5, w, w, f), ((1 << 22) + 1, 0, 0, 1.5, w, w, f), (2, 3, 0, 1.5, w, w, f), (2, -1, 0, 1.5, w, w, f),
+                 (2, 0, 2, 1.5, w, w, f), (2, 0, 0, 1.0, w, w, f), (2, 0, 0, 1.5, None, w, f), (2, 0, 0, 1.5, w, None, f),
+                 (2, 0, 0, 1.5, w, w, None)):
+        assert lib.icarus_face_check(*args) == EINVAL, args
