@@ -364,12 +364,12 @@ template <typename R> __device__ __forceinline__ void prim2cons(const R *w, R *u
 // final rounding: within one ulp of the correctly rounded root, almost always equal. s and y are kept
 // a little low, so that the sum errs downwards: the roots of 4^k (1 - 2^-53), just below a rounding
 // boundary, then come out right.
-// Zero, negative, subnormal and non-finite x take the library sqrt.
-__device__ __forceinline__ double sqrt_nr(double x)
+// Zero, negative, subnormal and non-finite x (not positive_normal) take the library sqrt.
+__device__ __forceinline__ bool positive_normal(double x) { return (unsigned int)__double2hiint(x) - 0x00100000u < 0x7fe00000u; }
+__device__ __forceinline__ double sqrt_normal(double x)
 {
     const int hi = __double2hiint(x);
     const unsigned int lo = (unsigned int)__double2loint(x);
-    if ((unsigned int)hi - 0x00100000u >= 0x7fe00000u) return sqrt(x);   // not positive and normal
     const int e = hi >> 20;
     const int k = (e - 1023) >> 1, odd = (e - 1023) & 1;
     const float mh = __int_as_float(((127 + odd) << 23) | ((hi & 0xfffff) << 3) | (int)(lo >> 29));
@@ -384,6 +384,7 @@ __device__ __forceinline__ double sqrt_nr(double x)
     const double h = __hiloint2double((((hb >> 23) + 895 - k) << 20) | ((hb & 0x7fffff) >> 3), hb << 29);
     return fma(h, fma(-s, s, x), s);
 }
+__device__ __forceinline__ double sqrt_nr(double x) { return positive_normal(x) ? sqrt_normal(x) : sqrt(x); }
 
 template <bool NR> __device__ __forceinline__ double root(double x) { return NR ? sqrt_nr(x) : sqrt(x); }
 template <bool NR> __device__ __forceinline__ float root(float x) { return sqrtf(x); }
@@ -664,15 +665,29 @@ __device__ __forceinline__ void tvdlf_paired(const float2 *w, int d, float gamma
     for (int v = 0; v < NV; ++v) f[v] = 0.5f * (F[v].x + F[v].y) - hc * (u[v].y - u[v].x);
 }
 
+// fast speed in double precision from a = gamma p, bb = B^2 and the normal field bn, in the rho-scaled form
+// c_f^2 rho = (S + sqrt(S^2 - 4 gamma p B_n^2)) / 2 with S = gamma p + B^2, so that 1/rho enters once. A
+// discriminant that is not positive and normal (S^2 outside the range of a double, or exactly degenerate
+// speeds) divides the terms by rho first, like fast_speed (a call in the place of the root's own slow path)
+static __device__ __noinline__ double fast_speed_scaled(double a, double bb, double bn, double irho)
+{
+    const double a2 = a * irho, s = fma(bb, irho, a2);
+    return sqrt_nr(half_r(s + sqrt_nr(clamp0_r(fma(s, s, -(quad_r(a2) * (bn * bn * irho)))))));
+}
+__device__ __forceinline__ double fast_speed_d(double a, double bb, double bn, double irho)
+{
+    const double S = a + bb, disc = fma(S, S, -(quad_r(a) * (bn * bn)));
+    if (!positive_normal(disc)) return fast_speed_scaled(a, bb, bn, irho);
+    return sqrt_nr(half_r(S + sqrt_normal(disc)) * irho);
+}
+
 // double-precision TVDLF with the fewest FP64 operations (the FP64 pipe is the bound): with the half
 // velocities h = v_n / 2 and the half speed c = c_max / 2, the combination (F_L + F_R)/2 -
 // c_max (U_R - U_L)/2 of a field carried by v_n is U_L (h_L + h_R) + (U_R - U_L)(h_R - c), two
 // operations after the difference, where the terms small against the flux stay small (no
 // cancellation of U (h + c) against U (h - c)); the B_n B / p_tot terms are added from the halved
-// normal field (exact halvings on the integer pipe). The fast speeds come from rho-scaled sums,
-// c_f^2 rho = (S + sqrt(S^2 - 4 gamma p B_n^2)) / 2 with S = gamma p + B^2, so that 1/rho enters once.
-// About 100 FP64 operations a face where the two sides' fluxes and their combination took 130; the nine
-// differences U_R - U_L go to the integer pipe (all 20 additions there: the integer pipe becomes the
+// normal field (exact halvings on the integer pipe). About 100 FP64 operations a face where the two
+// sides' fluxes and their combination took 130; the nine differences U_R - U_L go to the integer pipe (all 20 additions there: the integer pipe becomes the
 // bound, r / theta / phi flux 0.94 / 1.04 / 1.00 ms at 512 x 64 x 128 against 0.91 / 0.98 / 0.94).
 __device__ __forceinline__ void tvdlf_d(const double *wl, const double *wr, int d, double gamma, double igm1, double irl,
                                         double irr, double *f)
@@ -690,9 +705,7 @@ __device__ __forceinline__ void tvdlf_d(const double *wl, const double *wr, int 
         bv[s] = fma(w[5], w[1], fma(w[6], w[2], w[7] * w[3]));
         e[s] = fma(w[4], igm1, half_r(mv + bb));
         pt[s] = fma(0.5, bb, w[4]);
-        const double a = gamma * w[4], S = a + bb, bn = w[4 + n];
-        const double disc = clamp0_r(fma(S, S, -(quad_r(a) * (bn * bn))));
-        cs[s] = sqrt_nr(half_r(S + sqrt_nr(disc)) * (s ? irr : irl));
+        cs[s] = fast_speed_d(gamma * w[4], bb, w[4 + n], s ? irr : irl);
     }
     const double c = half_r(max_nonneg_r(abs_r(wl[n]) + cs[0], abs_r(wr[n]) + cs[1]));
     const double hl = half_r(wl[n]), hr = half_r(wr[n]), bl = half_r(wl[4 + n]), br = half_r(wr[4 + n]);
@@ -772,9 +785,8 @@ __device__ __forceinline__ void hll_d(const double *wl, const double *wr, int d,
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
         const double *w = s ? wr : wl;
-        const double bb = fma(w[5], w[5], fma(w[6], w[6], w[7] * w[7])), a = gamma * w[4], S = a + bb, bn = w[4 + n];
-        const double disc = clamp0_r(fma(S, S, -(quad_r(a) * (bn * bn))));
-        c[s] = sqrt_nr(half_r(S + sqrt_nr(disc)) * (s ? irr : irl));
+        const double bb = fma(w[5], w[5], fma(w[6], w[6], w[7] * w[7]));
+        c[s] = fast_speed_d(gamma * w[4], bb, w[4 + n], s ? irr : irl);
     }
     const double l0 = sub_i(wl[n], c[0]), l1 = sub_i(wr[n], c[1]), r0 = add_i(wl[n], c[0]), r1 = add_i(wr[n], c[1]);
     const double sl = less_i(l0, l1) ? l0 : l1, sr = less_i(r1, r0) ? r0 : r1;

@@ -103,3 +103,17 @@ def test_hll_nan_on_one_side(ic, d, mach):
     for q in range(16):
         (wl if q < 8 else wr)[q * 100:(q + 1) * 100, q % 8] = np.nan
     compare(ic, wl, wr, d, I.FLUX_HLL)
+
+
+@pytest.mark.parametrize("flux", [I.FLUX_TVDLF, I.FLUX_HLL])
+@pytest.mark.parametrize("k", [-450, -300, -260, -250, -240, 240, 251, 255, 260, 300, 450])
+def test_scaled_states(ic, flux, k):
+    """rho and p scaled by 4^k, B by 2^k leave the speeds as they are; the products gamma p + B^2 squared leave
+    the normal range at |k| = 256."""
+    rng = np.random.default_rng(20)
+    for d in range(3):
+        wl, wr = states(rng, 4000, 0.7), states(rng, 4000, 0.7)
+        for w in (wl, wr):
+            w[:, [0, 4]] *= 4.0 ** k
+            w[:, 5:8] *= 2.0 ** k
+        compare(ic, wl, wr, d, flux)
