@@ -489,7 +489,7 @@ __device__ __forceinline__ double vanleer_half(double a, double b, double s)
 // van Leer a b / (a + b); minmod min(|a|, |b|) / 2; monotonised central min(|a|, |b|, |a + b| / 4), with
 // magnitudes compared as integers and the exact halvings on the exponent (as FP64 arithmetic these
 // took about ten operations a field)
-static __device__ __noinline__ double quarter_slow(double x) { return 0.25 * x; }
+static __device__ __noinline__ double scale_slow(double x, double f) { return f * x; }
 __device__ __forceinline__ double half_slope(int lim, double a, double b)
 {
     if ((hi_bits(a) ^ hi_bits(b)) < 0 || is_zero(a) || is_zero(b)) return 0.0;
@@ -501,15 +501,18 @@ __device__ __forceinline__ double half_slope(int lim, double a, double b)
                              mb = (unsigned long long)(bh & 0x7fffffffu) << 32 | bl;
     unsigned long long m = ma < mb ? ma : mb;
     const unsigned int sign = ah & 0x80000000u;
-    if (lim == 0) return half_r(join_d((unsigned int)(m >> 32) | sign, (unsigned int)m));
+    const unsigned int mh = (unsigned int)(m >> 32), me = mh >> 20;
+    if (lim == 0) return me - 2u < 2045u ? join_d((mh - (1u << 20)) | sign, (unsigned int)m)
+                                         : scale_slow(join_d(mh | sign, (unsigned int)m), 0.5);
     double t = add_i(a, b);
     unsigned int th, tl;
     split_d(t, th, tl);
     const unsigned int e = (th >> 20) & 0x7ffu;
-    if (e == 0x7ffu) return t;                                   // NaN, or beyond the range
+    // NaN; a sum beyond the range: the smaller magnitude, unless its double is beyond the range too
+    if (e == 0x7ffu) return ((th << 12) | tl) != 0u || me >= 2046u ? t : join_d(mh | sign, (unsigned int)m);
     if (e >= 3u) th -= 2u << 20;
     else {
-        t = quarter_slow(t);
+        t = scale_slow(t, 0.25);
         split_d(t, th, tl);
     }
     const unsigned long long mt = (unsigned long long)(th & 0x7fffffffu) << 32 | tl;
