@@ -680,60 +680,109 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const float *__restrict__ 
 }
 
 // ---- normalisation, loss, correction, optimiser --------------------------------------------------
-// x[z][c] = (U[c][v] - mean[c][i]) / scale[c][i] for c < 8, 0 for c in [8, 16)
+// Conversions on the integer pipe (the FP64 pipe, which runs the hardware's, is the bound of these kernels).
+// narrow_d2f and widen_f2d flush magnitudes below the normal single-precision range, which the hardware
+// keeps: `low` takes how close a voxel's values came to one (below LOW_D / LOW_F: one is there), and such
+// a voxel is done again with the hardware conversions, in a call, so that the others share no code with it.
+// The scales of the divisions are converted once, when they are set.
+constexpr unsigned int LOW_D = 0x01800000u, LOW_F = 0x7fffffu;
+template <bool HW> __device__ __forceinline__ float narrow(double x, unsigned int &low)
+{
+    if (HW) return (float)x;
+    low = min(low, ((unsigned int)__double2hiint(x) & 0x7fffffffu) - 0x36900000u);   // 2^-150 <= |x| < 2^-126
+    return narrow_d2f(x);
+}
+template <bool HW> __device__ __forceinline__ double widen(float x, unsigned int &low)
+{
+    if (HW) return (double)x;
+    low = min(low, (__float_as_uint(x) & 0x7fffffffu) - 1u);                          // 0 < |x| < 2^-126
+    return widen_f2d(x);
+}
+
+__global__ void k_narrow_scales(int n, const double *__restrict__ a, const double *__restrict__ b, float *af, float *bf)
+{
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < n) { af[q] = (float)a[q]; bf[q] = (float)b[q]; }
+}
+
+// x[z][c] = (U[c][v] - mean[c][i]) / scale[c][i] for c < 8, 0 for c in [8, 16): (U - mean) in double, the
+// division by the scale in single precision (the result is BF16)
+template <bool HW>
+__device__ __forceinline__ bool norm_voxel(const double *__restrict__ U, long long N, const double *__restrict__ mean,
+                                           const float *__restrict__ scale, int n1, uint4 *d)
+{
+    uint32_t pk[4];
+    unsigned int low = ~0u;
+#pragma unroll
+    for (int c = 0; c < NV; c += 2) {
+        const float a = narrow<HW>(U[c * N] - mean[c * n1], low) / scale[c * n1];
+        const float b = narrow<HW>(U[(c + 1) * N] - mean[(c + 1) * n1], low) / scale[(c + 1) * n1];
+        pk[c / 2] = pack2(__float2bfloat16_rn(a), __float2bfloat16_rn(b));
+    }
+    d[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    d[1] = make_uint4(0u, 0u, 0u, 0u);                 // channels 8 .. 15 are zero padding
+    return low < LOW_D;
+}
+__device__ __noinline__ void norm_voxel_low(const double *U, long long N, const double *mean, const float *scale, int n1, uint4 *d)
+{
+    norm_voxel<true>(U, N, mean, scale, n1, d);
+}
 __global__ void k_norm_in(Geo g, const double *__restrict__ U, const double *__restrict__ mean,
-                          const double *__restrict__ scale, bf16 *x)
+                          const float *__restrict__ scale, bf16 *x)
 {
     const unsigned int v = blockIdx.x * blockDim.x + threadIdx.x;     // voxels < 2^31
     if (v >= (unsigned int)g.N) return;
     const unsigned int r = v / (unsigned int)g.n1;
     const int i = (int)(v % (unsigned int)g.n1), j = (int)(r % (unsigned int)g.n2), k = (int)(r / (unsigned int)g.n2);
-    // (U - mean) in double, the division by the scale in single precision (the result is BF16); conversions
-    // on the integer pipe (the FP64 pipe, which runs the hardware's, is the bound of these kernels)
-    uint32_t pk[8];
-#pragma unroll
-    for (int c = 0; c < NV; c += 2) {
-        const float a = narrow_d2f(U[c * g.N + v] - mean[c * g.n1 + i]) / narrow_d2f(scale[c * g.n1 + i]);
-        const float b = narrow_d2f(U[(c + 1) * g.N + v] - mean[(c + 1) * g.n1 + i]) / narrow_d2f(scale[(c + 1) * g.n1 + i]);
-        pk[c / 2] = pack2(__float2bfloat16_rn(a), __float2bfloat16_rn(b));
-    }
-#pragma unroll
-    for (int c = 4; c < 8; ++c) pk[c] = 0u;            // channels 8 .. 15 are zero padding
     uint4 *d = reinterpret_cast<uint4 *>(x + pidx(g, i, j, k) * 16);
-    d[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    d[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+    if (norm_voxel<false>(U + v, g.N, mean + i, scale + i, g.n1, d)) norm_voxel_low(U + v, g.N, mean + i, scale + i, g.n1, d);
 }
 
-// loss = mean over voxels and the 8 fields of (y - dU / oscale)^2; dy = its gradient
+// one voxel's part of the loss, mean over voxels and the 8 fields of (y - dU / oscale)^2, into s; dy = its
+// gradient; per element in single precision (the network's own precision), the sum in double
+template <bool HW>
+__device__ __forceinline__ bool mse_voxel(long long N, const float4 *yv, const double *__restrict__ dU,
+                                          const float *__restrict__ oscale, int n1, float4 *dv, double &s)
+{
+    const float norm = (float)(1.0 / (8.0 * (double)N));
+    float e[NV];
+    unsigned int low = ~0u, lowf = ~0u;
+    s = 0.0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float4 yy = yv[h];
+        const float ya[4] = {yy.x, yy.y, yy.z, yy.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = 4 * h + q;
+            e[c] = ya[q] - narrow<HW>(dU[c * N], low) / oscale[c * n1];
+            s += widen<HW>(e[c] * e[c], lowf);
+        }
+    }
+    s *= (double)norm;
+    dv[0] = make_float4(2.f * e[0] * norm, 2.f * e[1] * norm, 2.f * e[2] * norm, 2.f * e[3] * norm);
+    dv[1] = make_float4(2.f * e[4] * norm, 2.f * e[5] * norm, 2.f * e[6] * norm, 2.f * e[7] * norm);
+    dv[2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    dv[3] = make_float4(0.f, 0.f, 0.f, 0.f);
+    return low < LOW_D || lowf < LOW_F;
+}
+__device__ __noinline__ double mse_voxel_low(long long N, const float4 *yv, const double *dU, const float *oscale, int n1, float4 *dv)
+{
+    double s;
+    mse_voxel<true>(N, yv, dU, oscale, n1, dv, s);
+    return s;
+}
 __global__ void __launch_bounds__(256) k_mse(Geo g, const float *__restrict__ y, const double *__restrict__ dU,
-                                             const double *__restrict__ oscale, float *dy, double *loss)
+                                             const float *__restrict__ oscale, float *dy, double *loss)
 {
     __shared__ double red[8];
     const unsigned int v = blockIdx.x * blockDim.x + threadIdx.x;   // voxels < 2^31
     double s = 0.0;
     if (v < (unsigned int)g.N) {
         const int i = (int)(v % (unsigned int)g.n1);
-        // per element in single precision (the network's own precision), the sum in double
-        const float norm = (float)(1.0 / (8.0 * (double)g.N));
         const float4 *yv = reinterpret_cast<const float4 *>(y + (long long)v * 16);
         float4 *dv = reinterpret_cast<float4 *>(dy + (long long)v * 16);
-        float e[NV];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float4 yy = yv[h];
-            const float ya[4] = {yy.x, yy.y, yy.z, yy.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int c = 4 * h + q;
-                e[c] = ya[q] - narrow_d2f(dU[(long long)c * g.N + v]) / narrow_d2f(oscale[c * g.n1 + i]);
-                s += widen_f2d(e[c] * e[c]);
-            }
-        }
-        s *= (double)norm;
-        dv[0] = make_float4(2.f * e[0] * norm, 2.f * e[1] * norm, 2.f * e[2] * norm, 2.f * e[3] * norm);
-        dv[1] = make_float4(2.f * e[4] * norm, 2.f * e[5] * norm, 2.f * e[6] * norm, 2.f * e[7] * norm);
-        dv[2] = make_float4(0.f, 0.f, 0.f, 0.f);
-        dv[3] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (mse_voxel<false>(g.N, yv, dU + v, oscale + i, g.n1, dv, s)) s = mse_voxel_low(g.N, yv, dU + v, oscale + i, g.n1, dv);
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -745,7 +794,27 @@ __global__ void __launch_bounds__(256) k_mse(Geo g, const float *__restrict__ y,
     }
 }
 
+// whether one of the network's eight outputs of a voxel is below the normal range
+__device__ __forceinline__ bool low_outputs(const float *y)
+{
+    unsigned int low = ~0u;
+#pragma unroll
+    for (int f = 0; f < NV; ++f) low = min(low, (__float_as_uint(y[f]) & 0x7fffffffu) - 1u);
+    return low < LOW_F;
+}
+
 // correction in the solver's padded FP64 layout: U[c] += y[c] * oscale[c][i]
+template <bool HW>
+__device__ __forceinline__ void apply_voxel(const float *y, const double *__restrict__ oscale, int n1, double *U, long long nt)
+{
+    unsigned int low = ~0u;
+#pragma unroll
+    for (int f = 0; f < NV; ++f) U[f * nt] += widen<HW>(y[f], low) * oscale[f * n1];
+}
+__device__ __noinline__ void apply_voxel_low(const float *y, const double *oscale, int n1, double *U, long long nt)
+{
+    apply_voxel<true>(y, oscale, n1, U, nt);
+}
 __global__ void k_apply(Params P, Geo g, const float *__restrict__ y, const double *__restrict__ oscale, double *U)
 {
     long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -754,16 +823,29 @@ __global__ void k_apply(Params P, Geo g, const float *__restrict__ y, const doub
     const long long r = v / g.n1;
     const int j = (int)(r % g.n2), k = (int)(r / g.n2);
     const long long c = cidx(P, i, j, k);
-    for (int f = 0; f < NV; ++f) U[f * P.nt + c] += widen_f2d(y[v * 16 + f]) * oscale[f * g.n1 + i];
+    if (low_outputs(y + v * 16)) apply_voxel_low(y + v * 16, oscale + i, g.n1, U + c, P.nt);
+    else apply_voxel<false>(y + v * 16, oscale + i, g.n1, U + c, P.nt);
 }
 
+template <bool HW>
+__device__ __forceinline__ bool unpack_voxel(const float *y, const double *__restrict__ oscale, int n1, double *dU, long long N)
+{
+    unsigned int low = ~0u;
+#pragma unroll
+    for (int f = 0; f < NV; ++f) dU[f * N] = widen<HW>(y[f], low) * oscale[f * n1];
+    return low < LOW_F;
+}
+__device__ __noinline__ void unpack_voxel_low(const float *y, const double *oscale, int n1, double *dU, long long N)
+{
+    unpack_voxel<true>(y, oscale, n1, dU, N);
+}
 __global__ void k_unpack_dU(Geo g, const float *__restrict__ y, const double *__restrict__ oscale, double *dU)
 {
     const unsigned int v = blockIdx.x * blockDim.x + threadIdx.x;     // voxels < 2^31
     if (v >= (unsigned int)g.N) return;
     const int i = (int)(v % (unsigned int)g.n1);
-#pragma unroll
-    for (int f = 0; f < NV; ++f) dU[f * g.N + v] = widen_f2d(y[(long long)v * 16 + f]) * oscale[f * g.n1 + i];
+    const float *yv = y + (long long)v * 16;
+    if (unpack_voxel<false>(yv, oscale + i, g.n1, dU + v, g.N)) unpack_voxel_low(yv, oscale + i, g.n1, dU + v, g.N);
 }
 
 // one layer's weights, their moments, gradients and BF16 copies w[O][27][C] and wt[C][27][O]
@@ -1039,6 +1121,7 @@ struct icarus_closure {
     float *wpart;          // partial sums of the weight-gradient blocks
     float *y, *dy;         // [N][16]
     double *mean, *scale, *oscale, *loss, *upack;
+    float *scale_f, *oscale_f;   // the scales as the divisions take them
     float *grads = nullptr;   // [loss (2 floats) | dw, db of each layer]
     size_t n_grads = 0;
     int step = 0;
@@ -1163,9 +1246,11 @@ int icarus_closure_create(int n1, int n2, int n3, unsigned long long seed, void 
         c->mean = (double *)cl_alloc(c, 8 * n1 * 8);
         c->scale = (double *)cl_alloc(c, 8 * n1 * 8);
         c->oscale = (double *)cl_alloc(c, 8 * n1 * 8);
+        c->scale_f = (float *)cl_alloc(c, 8 * n1 * 4);
+        c->oscale_f = (float *)cl_alloc(c, 8 * n1 * 4);
         c->upack = (double *)cl_alloc(c, 8 * g.N * 8);
         c->wpart = (float *)cl_alloc(c, wgrad_part_floats() * 4);
-        ok = c->dpre && c->din && c->y && c->dy && c->mean && c->scale && c->oscale && c->loss && c->upack && c->wpart;
+        ok = c->dpre && c->din && c->y && c->dy && c->mean && c->scale && c->oscale && c->scale_f && c->oscale_f && c->loss && c->upack && c->wpart;
     }
     if (!ok) {
         for (void *p : c->allocs) cudaFree(p);
@@ -1195,6 +1280,8 @@ int icarus_closure_set_norm(icarus_closure *c, const double *in_mean, const doub
     CCK(cudaMemcpyAsync(c->mean, in_mean, n, cudaMemcpyHostToDevice, c->stream));
     CCK(cudaMemcpyAsync(c->scale, in_scale, n, cudaMemcpyHostToDevice, c->stream));
     CCK(cudaMemcpyAsync(c->oscale, out_scale, n, cudaMemcpyHostToDevice, c->stream));
+    k_narrow_scales<<<ccdiv(8LL * c->g.n1, 256), 256, 0, c->stream>>>(8 * c->g.n1, c->scale, c->oscale, c->scale_f, c->oscale_f);
+    CCK(cudaGetLastError());
     CCK(cudaStreamSynchronize(c->stream));
     c->have_norm = true;
     return ICARUS_OK;
@@ -1206,12 +1293,12 @@ int icarus_closure_train_step(icarus_closure *c, const double *U_in, const doubl
     if (!c->have_norm) return report_error(ICARUS_ESTATE, "set the normalisation first");
     cudaStream_t s = c->stream;
     const Geo g = c->g;
-    k_norm_in<<<ccdiv(g.N, 256), 256, 0, s>>>(g, U_in, c->mean, c->scale, c->act[0]);
+    k_norm_in<<<ccdiv(g.N, 256), 256, 0, s>>>(g, U_in, c->mean, c->scale_f, c->act[0]);
     k_pad_fill<bf16><<<ccdiv(g.NP, 256), 256, 0, s>>>(g, c->act[0], 16);
     forward(c);
     if (tc_map_failed()) return report_error(ICARUS_ECUDA, "tensor map encoding failed");
     CCK(cudaMemsetAsync(c->grads, 0, c->n_grads * 4, s));
-    k_mse<<<ccdiv(g.N, 256), 256, 0, s>>>(g, c->y, dU_target, c->oscale, c->dy, c->loss);
+    k_mse<<<ccdiv(g.N, 256), 256, 0, s>>>(g, c->y, dU_target, c->oscale_f, c->dy, c->loss);
     // layer 3 (linear): gradient from the loss; then ReLU layers with the mask of their output
     for (int l = 3; l >= 0; --l) {
         if (l == 3) launch_dpre(LO[l], g, c->dy, 0, nullptr, c->dpre, c->db[l], s);
@@ -1246,7 +1333,7 @@ int icarus_closure_predict(icarus_closure *c, const double *U_in, double *dU_out
     if (!c->have_norm) return report_error(ICARUS_ESTATE, "set the normalisation first");
     cudaStream_t s = c->stream;
     const Geo g = c->g;
-    k_norm_in<<<ccdiv(g.N, 256), 256, 0, s>>>(g, U_in, c->mean, c->scale, c->act[0]);
+    k_norm_in<<<ccdiv(g.N, 256), 256, 0, s>>>(g, U_in, c->mean, c->scale_f, c->act[0]);
     k_pad_fill<bf16><<<ccdiv(g.NP, 256), 256, 0, s>>>(g, c->act[0], 16);
     forward(c);
     if (tc_map_failed()) return report_error(ICARUS_ECUDA, "tensor map encoding failed");
@@ -1267,7 +1354,7 @@ int icarus_closure_apply(icarus_closure *c, icarus_ctx *ctx)
     CCK(cudaStreamSynchronize(c->stream));
     ctx->ops.pack(ctx->P, ctx->U, c->upack, s);
     const Geo g = c->g;
-    k_norm_in<<<ccdiv(g.N, 256), 256, 0, s>>>(g, c->upack, c->mean, c->scale, c->act[0]);
+    k_norm_in<<<ccdiv(g.N, 256), 256, 0, s>>>(g, c->upack, c->mean, c->scale_f, c->act[0]);
     k_pad_fill<bf16><<<ccdiv(g.NP, 256), 256, 0, s>>>(g, c->act[0], 16);
     cudaStream_t keep = c->stream;
     c->stream = s;
