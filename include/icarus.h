@@ -425,6 +425,13 @@ int icarus_restrict(icarus_ctx *fine, icarus_ctx *coarse);
 int icarus_conv3d_layer(int n1, int n2, int n3, int C, int O, int act, const float *x, const float *w,
                         const float *b, const float *g, float *y, float *dx, float *dw, float *db);
 
+/* The pre-activation gradient of a hidden layer as the training forms it, on host FP32 arrays with one ghost
+ * layer ([n3 + 2][n2 + 2][n1 + 2][O], O 16 or 32): dout the next layer's data gradient, whose ghost cells'
+ * values are added to the cells they copy, act the layer's activated output (rounded to BF16; the ReLU's
+ * mask) to dpre (BF16 values, zero ghosts) and the bias gradient db [O]. For checking the kernel against
+ * a reference. */
+int icarus_dpre_check(int n1, int n2, int n3, int O, const float *dout, const float *act, float *dpre, float *db);
+
 /* Largest grid (interior cells) icarus_cfl_dt_noalloc accepts: 16384 blocks of 256 cells. */
 #define ICARUS_NOALLOC_MAX_CELLS 4194304LL
 

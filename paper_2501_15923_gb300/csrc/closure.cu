@@ -12,7 +12,8 @@
 // (theta, phi) lines x C_in, K = padded positions split over blocks, operands transposed into
 // shared memory with movmatrix, blocks' partial sums reduced by a second kernel). Activations are stored
 // channels-last on a grid padded by one ghost layer; a pad kernel fills the ghosts (replicate /
-// circular) and a fold kernel adds ghost gradients back to the cells they copy (the adjoint).
+// circular); the ghost gradients are added back to the cells they copy (the adjoint) where the
+// pre-activation gradient of the layer below reads them.
 // Channel counts are padded to multiples of 16 (layer 0 input 8 -> 16 zero channels, layer 3
 // output 8 -> 16 with zero weights); the padding never carries a gradient.
 #include <cuda.h>
@@ -362,19 +363,42 @@ __global__ void k_pad_fill(Geo g, T *buf, int C)
     }
 }
 
-// add every ghost cell's gradient to the interior cell it copies (in place, interior = result)
-__global__ void k_pad_fold(Geo g, float *buf, int C)
+// the padding's adjoint: gradient of eight channels from c0 on of the interior cell (i, j, k) = padded cell q,
+// its own and those of the ghost cells that copy it: i - 1 / i + 1 at the ends of r, likewise theta, and
+// the periodic images of k
+__device__ __forceinline__ void folded(const Geo &g, const float *__restrict__ dout, int O, int c0, unsigned int q, int i, int j,
+                                       int k, float *d)
 {
-    long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= g.NP) return;
-    int ip = (int)(q % g.q1);
-    long long r = q / g.q1;
-    int jp = (int)(r % g.q2), kp = (int)(r / g.q2);
-    int i = ip - 1, j = jp - 1, k = kp - 1;
-    if (i >= 0 && i < g.n1 && j >= 0 && j < g.n2 && k >= 0 && k < g.n3) return;
-    int si = min(max(i, 0), g.n1 - 1), sj = min(max(j, 0), g.n2 - 1), sk = (k + g.n3) % g.n3;
-    long long src = pidx(g, si, sj, sk);
-    for (int c = 0; c < C; ++c) atomicAdd(&buf[src * C + c], buf[q * C + c]);
+    auto add = [&](long long cell, bool first) {
+        const float4 *src = reinterpret_cast<const float4 *>(dout + cell * O + c0);
+        const float4 x = src[0], y = src[1];
+        const float v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) d[e] = first ? v[e] : d[e] + v[e];
+    };
+    add(q, true);
+    if (i == 0 || i == g.n1 - 1 || j == 0 || j == g.n2 - 1 || k == 0 || k == g.n3 - 1)
+        for (int t = 0; t < 3; ++t) {
+            if ((t == 1 && k != 0) || (t == 2 && k != g.n3 - 1)) continue;
+            const int kk = t == 0 ? k : (t == 1 ? g.n3 : -1);
+            for (int jj = j == 0 ? -1 : j; jj <= (j == g.n2 - 1 ? g.n2 : j); ++jj)
+                for (int ii = i == 0 ? -1 : i; ii <= (i == g.n1 - 1 ? g.n1 : i); ++ii)
+                    if (ii != i || jj != j || kk != k) add(pidx(g, ii, jj, kk), false);
+        }
+}
+
+// the folded gradient of a layer's input in FP32, interior cells (the single-layer entry point)
+__global__ void k_fold(Geo g, const float *__restrict__ din, int C, float *dx)
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int G = C / 8, c0 = (int)(t % G) * 8;
+    const long long v = t / G;
+    if (v >= g.N) return;
+    const int i = (int)(v % g.n1), j = (int)(v / g.n1 % g.n2), k = (int)(v / g.n1 / g.n2);
+    float d[8];
+    folded(g, din, C, c0, (unsigned int)pidx(g, i, j, k), i, j, k, d);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) dx[v * C + c0 + e] = d[e];
 }
 
 // ---- gradient w.r.t. the pre-activation, bias gradient ------------------------------------------
@@ -402,26 +426,11 @@ __global__ void __launch_bounds__(256) k_dpre(Geo g, const float *__restrict__ d
         uint4 out = make_uint4(0u, 0u, 0u, 0u);
         if (i >= 0 && i < g.n1 && j >= 0 && j < g.n2 && k >= 0 && k < g.n3) {
             float d[8];
-            auto add = [&](long long cell, bool first) {
-                const float4 *src = reinterpret_cast<const float4 *>(dout + cell * O + c0);
-                const float4 x = src[0], y = src[1];
-                const float v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
-#pragma unroll
-                for (int e = 0; e < 8; ++e) d[e] = first ? v[e] : d[e] + v[e];
-            };
-            if (!dout_padded) add(((long long)k * g.n2 + j) * g.n1 + i, true);
+            if (dout_padded) folded(g, dout, O, c0, q, i, j, k, d);
             else {
-                add(q, true);
-                // the ghost cells that copy this one: i - 1 / i + 1 at the ends of r, likewise theta, and the
-                // periodic images of k
-                if (i == 0 || i == g.n1 - 1 || j == 0 || j == g.n2 - 1 || k == 0 || k == g.n3 - 1)
-                    for (int t = 0; t < 3; ++t) {
-                        if ((t == 1 && k != 0) || (t == 2 && k != g.n3 - 1)) continue;
-                        const int kk = t == 0 ? k : (t == 1 ? g.n3 : -1);
-                        for (int jj = j == 0 ? -1 : j; jj <= (j == g.n2 - 1 ? g.n2 : j); ++jj)
-                            for (int ii = i == 0 ? -1 : i; ii <= (i == g.n1 - 1 ? g.n1 : i); ++ii)
-                                if (ii != i || jj != j || kk != k) add(pidx(g, ii, jj, kk), false);
-                    }
+                const float4 *src = reinterpret_cast<const float4 *>(dout + (((long long)k * g.n2 + j) * g.n1 + i) * O + c0);
+                const float4 x = src[0], y = src[1];
+                d[0] = x.x; d[1] = x.y; d[2] = x.z; d[3] = x.w; d[4] = y.x; d[5] = y.y; d[6] = y.z; d[7] = y.w;
             }
             if (act_out) {
                 const uint4 a = *reinterpret_cast<const uint4 *>(act_out + (long long)q * O + c0);
@@ -1430,7 +1439,7 @@ int icarus_conv3d_layer(int n1, int n2, int n3, int C, int O, int act, const flo
     bf16 *din_ = (bf16 *)A(gg.NP * C * 2), *dout_ = (bf16 *)A(gg.NP * O * 2), *wb = (bf16 *)A(O * 27 * C * 2),
          *wt = (bf16 *)A(O * 27 * C * 2), *dpre = (bf16 *)A(gg.NP * O * 2);
     float *wf = (float *)A(O * 27 * C * 4), *bf = (float *)A(O * 4), *yf = (float *)A(gg.N * O * 4),
-          *gf = (float *)A(gg.N * O * 4), *dinf = (float *)A(gg.NP * C * 4), *dwf = (float *)A(O * 27 * C * 4),
+          *gf = (float *)A(gg.N * O * 4), *dinf = (float *)A(gg.NP * C * 4), *dxf = (float *)A(gg.N * C * 4), *dwf = (float *)A(O * 27 * C * 4),
           *dbf = (float *)A(O * 4), *wpart = (float *)A(wgrad_part_floats() * 4);
     int rc = ICARUS_OK;
     for (void *p : mem) if (!p) rc = report_error(ICARUS_ENOMEM, "allocation failed");
@@ -1459,7 +1468,7 @@ int icarus_conv3d_layer(int n1, int n2, int n3, int C, int O, int act, const flo
         } else {
             launch_dgrad_tc<32, 16>(gg, dpre, wt, dinf, 0);
         }
-        k_pad_fold<<<ccdiv(gg.NP, 256), 256>>>(gg, dinf, C);
+        k_fold<<<ccdiv(gg.N * (C / 8), 256), 256>>>(gg, dinf, C, dxf);
         cudaError_t e = cudaDeviceSynchronize();
         if (e != cudaSuccess) rc = report_error(ICARUS_ECUDA, cudaGetErrorString(e));
         else if (tc_timed_out()) rc = report_error(ICARUS_ETIMEOUT, "tensor-core forward: MMA completion wait expired");
@@ -1467,17 +1476,40 @@ int icarus_conv3d_layer(int n1, int n2, int n3, int C, int O, int act, const flo
             cudaMemcpy(y, yf, gg.N * O * 4, cudaMemcpyDeviceToHost);
             cudaMemcpy(dw, dwf, O * 27 * C * 4, cudaMemcpyDeviceToHost);
             cudaMemcpy(db, dbf, O * 4, cudaMemcpyDeviceToHost);
-            std::vector<float> hd(gg.NP * C);
-            cudaMemcpy(hd.data(), dinf, hd.size() * 4, cudaMemcpyDeviceToHost);
-            for (int k = 0; k < n3; ++k)
-                for (int j = 0; j < n2; ++j)
-                    for (int i = 0; i < n1; ++i)
-                        for (int c = 0; c < C; ++c)
-                            dx[(((size_t)k * n2 + j) * n1 + i) * C + c] = hd[pidx(gg, i, j, k) * C + c];
+            cudaMemcpy(dx, dxf, gg.N * C * 4, cudaMemcpyDeviceToHost);
         }
     }
     for (void *p : mem) cudaFree(p);
     return rc;
+}
+
+int icarus_dpre_check(int n1, int n2, int n3, int O, const float *dout, const float *act, float *dpre, float *db)
+{
+    if (n1 < 1 || n2 < 1 || n3 < 1 || (O != 16 && O != 32) || !dout || !act || !dpre || !db)
+        return report_error(ICARUS_EINVAL, "n1, n2, n3 >= 1, O 16 or 32, host arrays");
+    const Geo g = make_geo(n1, n2, n3);
+    if (g.NP >= (1LL << 31) / 32) return report_error(ICARUS_EINVAL, "grid too large for the check");
+    const size_t n = (size_t)g.NP * O;
+    float *d = nullptr, *b = nullptr;
+    bf16 *h = nullptr;                                 // activation, then dpre
+    std::vector<bf16> a(n);
+    for (size_t q = 0; q < n; ++q) a[q] = __float2bfloat16_rn(act[q]);
+    cudaError_t e = cudaMalloc(&d, n * 4);
+    if (e == cudaSuccess) e = cudaMalloc(&b, O * 4);
+    if (e == cudaSuccess) e = cudaMalloc(&h, 2 * n * 2);
+    if (e == cudaSuccess) e = cudaMemcpy(d, dout, n * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(h, a.data(), n * 2, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(b, 0, O * 4);
+    if (e == cudaSuccess) {
+        launch_dpre(O, g, d, 1, h, h + n, b, 0);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(a.data(), h + n, n * 2, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(db, b, O * 4, cudaMemcpyDeviceToHost);
+    for (size_t q = 0; q < n; ++q) dpre[q] = __bfloat162float(a[q]);
+    cudaFree(d); cudaFree(b); cudaFree(h);
+    if (e != cudaSuccess) return report_error(ICARUS_ECUDA, cudaGetErrorString(e));
+    return ICARUS_OK;
 }
 
 }  // extern "C"

@@ -98,6 +98,7 @@ SIGNATURES = {
     "icarus_closure_weights": (C.c_int, [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_int]),
     "icarus_restrict": (C.c_int, [C.c_void_p, C.c_void_p]),
     "icarus_conv3d_layer": (C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int] + [C.c_void_p] * 8),
+    "icarus_dpre_check": (C.c_int, [C.c_int] * 4 + [C.c_void_p] * 4),
     "icarus_cfl_dt_noalloc": (C.c_int, [C.POINTER(icarus_grid), C.c_double, C.c_double, C.c_void_p, C.c_void_p, C.c_void_p]),
     "icarus_fma_rate": (C.c_int, [C.c_int, C.c_int, C.c_int, C.c_longlong, C.POINTER(C.c_double), C.POINTER(C.c_double)]),
     "icarus_last_error": (C.c_char_p, []),

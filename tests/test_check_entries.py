@@ -28,3 +28,11 @@ def test_face_check(lib):
                  (2, 0, 2, 1.5, w, w, f), (2, 0, 0, 1.0, w, w, f), (2, 0, 0, 1.5, None, w, f), (2, 0, 0, 1.5, w, None, f),
                  (2, 0, 0, 1.5, w, w, None)):
         assert lib.icarus_face_check(*args) == EINVAL, args
+
+
+def test_dpre_check(lib):
+    a = (C.c_float * (27 * 32))()
+    for args in ((0, 1, 1, 32, a, a, a, a), (1, 1, 0, 32, a, a, a, a), (1, 1, 1, 8, a, a, a, a), (4096, 4096, 4, 32, a, a, a, a),
+                 (1, 1, 1, 32, None, a, a, a), (1, 1, 1, 32, a, None, a, a), (1, 1, 1, 32, a, a, None, a),
+                 (1, 1, 1, 32, a, a, a, None)):
+        assert lib.icarus_dpre_check(*args) == EINVAL, args
