@@ -283,6 +283,11 @@ int icarus_scales(icarus_ctx *ctx, double *s);
 /* Number of kernel launches one step makes (for launch accounting). */
 int icarus_launches_per_step(icarus_ctx *ctx);
 
+/* Number of kernel launches captured into the context's graphs since its creation (for launch accounting:
+ * a step replays graphs, which are captured when a call first needs them after a change of the boundary
+ * tables' sizes or of the registered probes). 0 for NULL. */
+long long icarus_captured_launches(icarus_ctx *ctx);
+
 /* The cudaStream_t the context runs on (for events and ordering with other work). */
 void *icarus_get_stream(icarus_ctx *ctx);
 

@@ -147,6 +147,7 @@ void drop_graph(icarus_ctx *c)
     if (c->graph) cudaGraphExecDestroy(c->graph);
     if (c->graph_k) cudaGraphExecDestroy(c->graph_k);
     c->graph = c->graph_k = nullptr;
+    c->graph_steps = 0;
     c->p_version++;
 }
 
@@ -390,7 +391,6 @@ int count_launches(const icarus_ctx *c)
 
 int build_graph(icarus_ctx *c)
 {
-    drop_graph(c);
     cudaGraph_t g;
     CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     enqueue_step(c, c->stream);
@@ -399,22 +399,26 @@ int build_graph(icarus_ctx *c)
     e = cudaGraphInstantiate(&c->graph, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return fail(ICARUS_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
-    c->launches_per_step = count_launches(c);
+    c->captured += count_launches(c);
     return ICARUS_OK;
 }
 
 // STEPS_K steps in one graph: one launch instead of STEPS_K (no gap between the steps), and each step's probe
 // kernel, one block bound by latency, runs on a branch beside the next step's kernels up to its second
-// update. 20 steps with probes at 60 x 16 x 32: 183 -> 175 us a step, 300 x 33 x 65 FP32: 194 -> 185
-constexpr int STEPS_K = 4;
+// update. 20 steps with probes at 60 x 16 x 32: 183 -> 175 us a step, 300 x 33 x 65 FP32: 194 -> 185.
+// Building it takes 115-140 us against 46-58 for the one-step graph, and a launch saves about 35, so it is
+// built once the steps of the present tables and probes reach STEPS_K_FROM: a program that changes its tables
+// after every few steps would pay for it each time (4 MIXED steps at 60 x 16 x 32 after a change: 404 us
+// with both graphs built, 304 with the one that is launched)
+constexpr int STEPS_K = 4, STEPS_K_FROM = 16;
 
 int build_graph_k(icarus_ctx *c)
 {
     const bool probes = c->P.n_probes > 0;
-    if (probes && !c->side) {
-        CK(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
-        CK(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-        CK(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+    if (probes) {
+        if (!c->side) CK(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+        if (!c->ev_fork) CK(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
+        if (!c->ev_join) CK(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
     }
     cudaGraph_t g;
     CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
@@ -437,6 +441,7 @@ int build_graph_k(icarus_ctx *c)
     if (e2 == cudaSuccess) cudaGraphDestroy(g);
     if (e != cudaSuccess || e2 != cudaSuccess)
         return fail(ICARUS_ECUDA, "graph capture: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
+    c->captured += (long long)STEPS_K * count_launches(c);
     return ICARUS_OK;
 }
 
@@ -729,15 +734,18 @@ int icarus_step(icarus_ctx *c, int n)
         const int st = *(volatile int *)c->hstatus;
         if (st) return status_fail(st);
     }
-    if (!c->graph) {
+    // only the graphs that this call launches are built
+    if (c->graph_steps < STEPS_K_FROM) c->graph_steps = n < STEPS_K_FROM ? c->graph_steps + n : n;
+    bool many = n >= STEPS_K && (c->graph_k || c->graph_steps >= STEPS_K_FROM);
+    if (many && !c->graph_k && build_graph_k(c) != ICARUS_OK) {
+        cudaGetLastError();
+        many = false;                                      // the steps one by one then
+    }
+    if ((many ? n % STEPS_K : n) > 0 && !c->graph) {
         int rc = build_graph(c);
         if (rc) return rc;
     }
-    if (n >= STEPS_K && !c->graph_k) {
-        int rc = build_graph_k(c);
-        if (rc) return rc;
-    }
-    for (; n >= STEPS_K; n -= STEPS_K) CK(cudaGraphLaunch(c->graph_k, c->stream));
+    for (; many && n >= STEPS_K; n -= STEPS_K) CK(cudaGraphLaunch(c->graph_k, c->stream));
     for (int q = 0; q < n; ++q) CK(cudaGraphLaunch(c->graph, c->stream));
     return ICARUS_OK;
 }
@@ -1100,6 +1108,8 @@ int icarus_launches_per_step(icarus_ctx *c)
     if (!c) return fail(ICARUS_EINVAL, "NULL context");
     return count_launches(c);
 }
+
+long long icarus_captured_launches(icarus_ctx *c) { return c ? c->captured : 0; }
 
 void *icarus_get_stream(icarus_ctx *c) { return c ? (void *)c->stream : nullptr; }
 

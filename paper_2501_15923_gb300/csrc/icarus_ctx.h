@@ -32,11 +32,12 @@ struct icarus_ctx {
     bool have_state = false, have_boundary = false;
     cudaGraphExec_t graph = nullptr;       // one step
     cudaGraphExec_t graph_k = nullptr;     // several steps, each step's probes beside the next step
+    int graph_steps = 0;                   // steps since the graphs were dropped (as far as it matters)
+    long long captured = 0;                // kernel launches captured into graphs so far
     cudaStream_t side = nullptr;           // (captured only) the probes' branch and its fork and join
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     long long ring_tail = 0;
     double t0, p0, b0, omega_code, gm_code;
-    int launches_per_step = 0;
     int p_version = 0;      // bumped whenever P changes (the batched form re-reads it)
     std::vector<double> colvec_host;
 };

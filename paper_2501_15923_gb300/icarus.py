@@ -74,6 +74,7 @@ SIGNATURES = {
     "icarus_face_check": (C.c_int, [C.c_int, C.c_int, C.c_int, C.c_double, C.c_void_p, C.c_void_p, C.c_void_p]),
     "icarus_scales": (C.c_int, [C.c_void_p, C.c_void_p]),
     "icarus_launches_per_step": (C.c_int, [C.c_void_p]),
+    "icarus_captured_launches": (C.c_longlong, [C.c_void_p]),
     "icarus_get_stream": (C.c_void_p, [C.c_void_p]),
     "icarus_time_kernels": (C.c_int, [C.c_void_p, C.c_int, C.c_void_p]),
     "icarus_batch_init": (C.c_int, [C.c_int, C.c_void_p, C.c_double, C.c_double, C.POINTER(icarus_options), C.POINTER(C.c_void_p)]),

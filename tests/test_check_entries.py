@@ -36,3 +36,7 @@ def test_dpre_check(lib):
                  (1, 1, 1, 32, None, a, a, a), (1, 1, 1, 32, a, None, a, a), (1, 1, 1, 32, a, a, None, a),
                  (1, 1, 1, 32, a, a, a, None)):
         assert lib.icarus_dpre_check(*args) == EINVAL, args
+
+
+def test_captured_launches(lib):
+    assert lib.icarus_captured_launches(None) == 0
