@@ -1110,7 +1110,8 @@ void launch_dgrad(int l, Geo g, const bf16 *dpre, const bf16 *wt, float *din, cu
 void launch_dpre(int O, Geo g, const float *dout, int padded, const bf16 *act, bf16 *dpre, float *db, cudaStream_t s)
 {
     const long long want = (g.NP * (O / 8) + 255) / 256;
-    const unsigned int nb = (unsigned int)(want < 152 * 8 ? want : 152 * 8);
+    const int most = 8 * sm_count();
+    const unsigned int nb = (unsigned int)(want < most ? want : most);
     if (O == 32) k_dpre<32><<<nb, 256, 0, s>>>(g, dout, padded, act, dpre, db);
     else k_dpre<16><<<nb, 256, 0, s>>>(g, dout, padded, act, dpre, db);
 }

@@ -522,8 +522,8 @@ __device__ __forceinline__ double half_slope(int lim, double a, double b)
 
 // half the limited slope in single precision. van Leer 2 a b / (a + b) as the product with the hardware
 // reciprocal, which is what the approximate division gives for 2^-126 <= |a + b| < 2^126 (the same bits)
-// without its range handling; above, where 2 a b only stays finite for a slope negligible against a + b,
-// the slope is 0
+// without its range handling; above, the reciprocal flushes to 0 and the slope is 0 (NaN where 2 a b is
+// infinite), as with that division
 __device__ __forceinline__ float half_slope(int lim, float a, float b)
 {
     if (lim != 1) return 0.5f * limiter<float>(lim, a, b);
@@ -690,8 +690,9 @@ __device__ __forceinline__ double fast_speed_d(double a, double bb, double bn, d
 // operations after the difference, where the terms small against the flux stay small (no
 // cancellation of U (h + c) against U (h - c)); the B_n B / p_tot terms are added from the halved
 // normal field (exact halvings on the integer pipe). About 100 FP64 operations a face where the two
-// sides' fluxes and their combination took 130; the nine differences U_R - U_L go to the integer pipe (all 20 additions there: the integer pipe becomes the
-// bound, r / theta / phi flux 0.94 / 1.04 / 1.00 ms at 512 x 64 x 128 against 0.91 / 0.98 / 0.94).
+// sides' fluxes and their combination took 130; the nine differences U_R - U_L go to the integer pipe (all
+// 20 additions there: the integer pipe becomes the bound, r / theta / phi flux 0.94 / 1.04 / 1.00 ms at 512 x
+// 64 x 128 against 0.91 / 0.98 / 0.94).
 __device__ __forceinline__ void tvdlf_d(const double *wl, const double *wr, int d, double gamma, double igm1, double irl,
                                         double irr, double *f)
 {
@@ -842,51 +843,51 @@ __device__ __forceinline__ void riemann(const R *wl, const R *wr, int d, int flu
     if constexpr (sizeof(R) == 8 && !HD) {
         if (flux == 0) tvdlf_d(wl, wr, d, gamma, igm1, irl, irr, f);
         else hll_d(wl, wr, d, gamma, igm1, irl, irr, f);
-        return;
-    }
-    R ul[NV], ur[NV];
-    prim2cons(wl, ul, igm1);
-    prim2cons(wr, ur, igm1);
-    R cl = fast_speed<R, true>(wl, irl, d, gamma), cr = fast_speed<R, true>(wr, irr, d, gamma);
-    R fl[NV], fr[NV];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        const R *w = s ? wr : wl;
-        const R *u = s ? ur : ul;
-        R *ff = s ? fr : fl;
-        R vn = w[1 + d], bn = w[5 + d];
-        R bb = w[5] * w[5] + w[6] * w[6] + w[7] * w[7];
-        R bv = w[5] * w[1] + w[6] * w[2] + w[7] * w[3];
-        R pt = w[4] + R(0.5) * bb;
-        ff[RHO] = u[RHO] * vn;
-        ff[M1] = u[M1] * vn - w[5] * bn;
-        ff[M2] = u[M2] * vn - w[6] * bn;
-        ff[M3] = u[M3] * vn - w[7] * bn;
-        ff[M1 + d] += pt;
-        ff[EN] = (u[EN] + pt) * vn - bn * bv;
-        ff[B1] = vn * w[5] - bn * w[1];
-        ff[B2] = vn * w[6] - bn * w[2];
-        ff[B3] = vn * w[7] - bn * w[3];
-        // the normal component v_n B_n - B_n v_n is exactly zero (the two products are equal; with
-        // a fused multiply-add it would come out as the product's rounding error instead)
-        ff[B1 + d] = R(0);
-    }
-    if constexpr (HD) {
-        (void)flux;
-        hlld<R>(wl, wr, ul, ur, fl, fr, cl, cr, d, f);
     } else {
-        R sl = rmin(wl[1 + d] - cl, wr[1 + d] - cr);
-        R sr = rmax(wl[1 + d] + cl, wr[1 + d] + cr);
-        if (sl >= R(0)) {
+        R ul[NV], ur[NV];
+        prim2cons(wl, ul, igm1);
+        prim2cons(wr, ur, igm1);
+        R cl = fast_speed<R, true>(wl, irl, d, gamma), cr = fast_speed<R, true>(wr, irr, d, gamma);
+        R fl[NV], fr[NV];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) f[v] = fl[v];
-        } else if (sr <= R(0)) {
-#pragma unroll
-            for (int v = 0; v < NV; ++v) f[v] = fr[v];
+        for (int s = 0; s < 2; ++s) {
+            const R *w = s ? wr : wl;
+            const R *u = s ? ur : ul;
+            R *ff = s ? fr : fl;
+            R vn = w[1 + d], bn = w[5 + d];
+            R bb = w[5] * w[5] + w[6] * w[6] + w[7] * w[7];
+            R bv = w[5] * w[1] + w[6] * w[2] + w[7] * w[3];
+            R pt = w[4] + R(0.5) * bb;
+            ff[RHO] = u[RHO] * vn;
+            ff[M1] = u[M1] * vn - w[5] * bn;
+            ff[M2] = u[M2] * vn - w[6] * bn;
+            ff[M3] = u[M3] * vn - w[7] * bn;
+            ff[M1 + d] += pt;
+            ff[EN] = (u[EN] + pt) * vn - bn * bv;
+            ff[B1] = vn * w[5] - bn * w[1];
+            ff[B2] = vn * w[6] - bn * w[2];
+            ff[B3] = vn * w[7] - bn * w[3];
+            // the normal component v_n B_n - B_n v_n is exactly zero (the two products are equal; with
+            // a fused multiply-add it would come out as the product's rounding error instead)
+            ff[B1 + d] = R(0);
+        }
+        if constexpr (HD) {
+            (void)flux;
+            hlld<R>(wl, wr, ul, ur, fl, fr, cl, cr, d, f);
         } else {
-            R idn = R(1) / (sr - sl);
+            R sl = rmin(wl[1 + d] - cl, wr[1 + d] - cr);
+            R sr = rmax(wl[1 + d] + cl, wr[1 + d] + cr);
+            if (sl >= R(0)) {
 #pragma unroll
-            for (int v = 0; v < NV; ++v) f[v] = (sr * fl[v] - sl * fr[v] + sl * sr * (ur[v] - ul[v])) * idn;
+                for (int v = 0; v < NV; ++v) f[v] = fl[v];
+            } else if (sr <= R(0)) {
+#pragma unroll
+                for (int v = 0; v < NV; ++v) f[v] = fr[v];
+            } else {
+                R idn = R(1) / (sr - sl);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) f[v] = (sr * fl[v] - sl * fr[v] + sl * sr * (ur[v] - ul[v])) * idn;
+            }
         }
     }
 }

@@ -493,10 +493,18 @@ k_flux_march(Params P, const float *__restrict__ W, float *__restrict__ F, int L
     }
 }
 
+// multiprocessors of the current device
+inline int sm_count()
+{
+    int dev = 0, sms = 0;
+    const bool ok = cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+    return ok && sms > 0 ? sms : 152;
+}
+
 // faces a thread marches through: 16, fewer (4 at least) while the chunks do not give every SM 48 warps
 inline int march_length(long long columns, int faces)
 {
-    const long long warps = (columns + 31) / 32, want = (152LL * 48 + warps - 1) / warps;
+    const long long warps = (columns + 31) / 32, want = (48LL * sm_count() + warps - 1) / warps;
     const long long lo = (faces + 15) / 16, hi = (faces + 3) / 4;
     const long long chunks = want < lo ? lo : (want < hi ? want : hi);
     return (int)((faces + chunks - 1) / chunks);
@@ -513,14 +521,15 @@ template <int D, int BX, int BY> __host__ __device__ inline void flux_tiles(cons
 // Tile shape and resident blocks per SM. FP64 (TVDLF / HLL): the FP64 and integer pipes are the bound,
 // so small blocks of 128 threads, which drift apart and keep both busy: r faces along the 32 lanes of a
 // warp (no block barrier), theta / phi faces in tiles of 8 x 16 (16 x 16: 1.08 / 1.05 ms against 0.98 /
-// 0.94 at 512 x 64 x 128); six blocks at 80 registers (five: 1.01 against 0.94 ms). Single precision: 40
-// registers (6 blocks of 256, 12 of 128; a few bytes of spills) instead of 48, measured 3-7 % faster
-// per flux kernel (issue-bound, latency-limited at 53-56 % warps active). No constraint for HLLD.
+// 0.94 at 512 x 64 x 128); six blocks at 80 registers (five: 1.01 against 0.94 ms). Single precision (r faces
+// of the separate sequence; theta and phi march): 40 registers (12 blocks of 128; a few bytes of spills)
+// instead of 48, measured 3-7 % faster (issue-bound, latency-limited at 53-56 % warps active). No
+// constraint for HLLD and GLM (HD).
 template <int D, typename TW, bool HD> struct FluxShape {
     static constexpr bool d = sizeof(TW) == 8 && !HD;
     static constexpr int BX = D == 0 ? (d ? 32 : 128) : (d ? 8 : 16);
     static constexpr int BY = D == 0 ? (d ? 4 : 1) : 16;
-    static constexpr int MINB = d ? 6 : (!HD ? (D == 0 ? 12 : 6) : 1);
+    static constexpr int MINB = d ? 6 : (HD ? 1 : 12);
 };
 
 template <int D, typename TW, bool HD = false>
@@ -1543,15 +1552,15 @@ __global__ void k_unpack(Params P, TS *__restrict__ U, const double *__restrict_
 
 // ---------------------------------------------------------------------------------------------
 // for A ascending arrays at once (32 samples of each a round, called by a whole warp): the largest q in
-// [0, n[a]) with x[a][q stride] <= v[a]; below[a]: there is none (q = 0)
+// [0, n[a]) with x[a][q stride] <= v[a], 0 if there is none
 template <int A> __device__ __forceinline__ void warp_search(const double *const *x, int stride, const int *size,
-                                                             const double *v, int *q, bool *below)
+                                                             const double *v, int *q)
 {
     const int lane = threadIdx.x & 31;
     int n[A], top = 0;
 #pragma unroll
-    for (int a = 0; a < A; ++a) { q[a] = 0; n[a] = size[a]; below[a] = false; top = max(top, n[a]); }
-    for (bool first = true; first || top > 1; first = false) {
+    for (int a = 0; a < A; ++a) { q[a] = 0; n[a] = size[a]; top = max(top, n[a]); }
+    while (top > 1) {
         bool le[A];
         int step[A];
 #pragma unroll
@@ -1564,7 +1573,6 @@ template <int A> __device__ __forceinline__ void warp_search(const double *const
 #pragma unroll
         for (int a = 0; a < A; ++a) {
             const int c = __popc(__ballot_sync(0xffffffffu, le[a]));
-            if (first) below[a] = c == 0;
             const int last = max(c, 1) - 1;
             q[a] += last * step[a];
             n[a] = min(step[a], n[a] - last * step[a]);
@@ -1592,8 +1600,7 @@ __device__ __forceinline__ void probe_warp(const Params &P, const TW *__restrict
     else if (tsi >= kn[(long long)(K - 1) * 4]) { a = K - 2; w = 1.0; }
     else {
         const int sz = K - 1;
-        bool below;
-        warp_search<1>(&kn, 4, &sz, &tsi, &a, &below);   // largest a with kn[a] <= tsi, a <= K-2
+        warp_search<1>(&kn, 4, &sz, &tsi, &a);           // largest a with kn[a] <= tsi, a <= K-2
         w = __ddiv_rn(__dsub_rn(tsi, kn[a * 4]), __dsub_rn(kn[(a + 1) * 4], kn[a * 4]));
     }
     const int b = K == 1 ? 0 : a + 1;
@@ -1613,8 +1620,7 @@ __device__ __forceinline__ void probe_warp(const Params &P, const TW *__restrict
     const double *const x[3] = {xc, yc, zc}, v[3] = {r, th, ph};
     const int size[3] = {max(n1 - 1, 1), max(n2 - 1, 1), n3};
     int ijk[3];
-    bool below[3];
-    warp_search<3>(x, 1, size, v, ijk, below);
+    warp_search<3>(x, 1, size, v, ijk);
     const int i = ijk[0], j = ijk[1], k = zc[0] > ph ? n3 - 1 : ijk[2];
     const double phk = zc[0] > ph ? __dsub_rn(zc[n3 - 1], TWO_PI) : zc[k];
     double wr = n1 > 1 ? (r - xc[i]) / (xc[i + 1] - xc[i]) : 0.0;
