@@ -489,7 +489,15 @@ __device__ __forceinline__ double vanleer_half(double a, double b, double s)
 // van Leer a b / (a + b); minmod min(|a|, |b|) / 2; monotonised central min(|a|, |b|, |a + b| / 4), with
 // magnitudes compared as integers and the exact halvings on the exponent (as FP64 arithmetic these
 // took about ten operations a field)
-static __device__ __noinline__ double scale_slow(double x, double f) { return f * x; }
+static __device__ __noinline__ double half_slow(double x) { return 0.5 * x; }
+// the monotonised central slope of the smaller difference x and the sum t where a quarter of t leaves the
+// normal range, t is beyond the range (x then, unless twice x is too) or NaN
+static __device__ __noinline__ double mc_slow(double x, double t)
+{
+    if (isinf(t)) return fabs(x) < 0x1p1023 ? x : t;
+    const double q = 0.25 * t;
+    return fabs(x) < fabs(q) ? x : q;
+}
 __device__ __forceinline__ double half_slope(int lim, double a, double b)
 {
     if ((hi_bits(a) ^ hi_bits(b)) < 0 || is_zero(a) || is_zero(b)) return 0.0;
@@ -503,18 +511,12 @@ __device__ __forceinline__ double half_slope(int lim, double a, double b)
     const unsigned int sign = ah & 0x80000000u;
     const unsigned int mh = (unsigned int)(m >> 32), me = mh >> 20;
     if (lim == 0) return me - 2u < 2045u ? join_d((mh - (1u << 20)) | sign, (unsigned int)m)
-                                         : scale_slow(join_d(mh | sign, (unsigned int)m), 0.5);
-    double t = add_i(a, b);
+                                         : half_slow(join_d(mh | sign, (unsigned int)m));
+    const double t = add_i(a, b);
     unsigned int th, tl;
     split_d(t, th, tl);
-    const unsigned int e = (th >> 20) & 0x7ffu;
-    // NaN; a sum beyond the range: the smaller magnitude, unless its double is beyond the range too
-    if (e == 0x7ffu) return ((th << 12) | tl) != 0u || me >= 2046u ? t : join_d(mh | sign, (unsigned int)m);
-    if (e >= 3u) th -= 2u << 20;
-    else {
-        t = scale_slow(t, 0.25);
-        split_d(t, th, tl);
-    }
+    if (((th >> 20) & 0x7ffu) - 3u >= 2044u) return mc_slow(join_d(mh | sign, (unsigned int)m), t);
+    th -= 2u << 20;
     const unsigned long long mt = (unsigned long long)(th & 0x7fffffffu) << 32 | tl;
     m = mt < m ? mt : m;
     return join_d((unsigned int)(m >> 32) | sign, (unsigned int)m);
