@@ -244,8 +244,8 @@ int icarus_time(icarus_ctx *ctx, double *t, double *dt);
 
 /* Check of the square root and the reciprocal that the FP64 kernels use in place of the library's
  * correctly rounded ones (the fast-speed roots in the Riemann flux; the reciprocals of the face
- * densities, of the van Leer slope sums and of rho): single-precision estimates refined by two
- * Newton steps, within one ulp of the correctly rounded results. For the n host values x,
+ * densities and of rho): single-precision estimates carried to 43 bits and finished by one Newton
+ * step, within one ulp of the correctly rounded results. For the n host values x,
  * y[4i .. 4i + 3] receive that root of x[i], the library sqrt, that reciprocal and the library
  * 1 / x[i]. Synchronous; a temporary device buffer. EINVAL for n outside [1, 2^24] or NULL. */
 int icarus_math_check(int n, const double *x, double *y);

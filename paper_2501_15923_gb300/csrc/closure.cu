@@ -10,7 +10,7 @@
 // memory, operands brought into shared memory by the tensor memory accelerator); the weight
 // gradient on the same tensor cores (rows = the three r shifts x C_out, columns = the nine
 // (theta, phi) lines x C_in, K = padded positions split over blocks, operands transposed into
-// shared memory with movmatrix, blocks' partial sums reduced by a second kernel). Activations are stored
+// shared memory by ldmatrix.trans, blocks' partial sums reduced by a second kernel). Activations are stored
 // channels-last on a grid padded by one ghost layer; a pad kernel fills the ghosts (replicate /
 // circular); the ghost gradients are added back to the cells they copy (the adjoint) where the
 // pre-activation gradient of the layer below reads them.

@@ -286,7 +286,12 @@ __device__ __forceinline__ void bnd23_cell(const Params &P, TS *__restrict__ U, 
 // consecutive r. Must be called by every thread of the block (it synchronises the block).
 // GLM (template flag, psi of type TP): psi is reconstructed alongside (cell and upper-face values
 // of the neighbour in sQW / sQP), and after the Riemann flux the (B_n, psi) star state replaces
-// the normal-field flux by psi* and writes c_h^2 B_n* to FP (the GLM div-B control's face step)
+// the normal-field flux by psi* and writes c_h^2 B_n* to FP (the GLM div-B control's face step).
+// In double (HLLD, GLM, the batched phases and persistent form) the half slopes are the integer-pipe ones:
+// a step at 256 x 32 x 64 with HLLD 2.96 -> 2.71 ms (van Leer), 3.34 -> 2.58 (MC), with GLM 2.10 -> 1.64;
+// plain FP64 slopes 2.82 / 3.21 / 1.82. Unrolled: a loop over the fields as in flux_tile_d takes 2.91 with
+// HLLD and 1.48 with GLM (1.64 unrolled), but at 60 x 16 x 32 it is the slower one with both (HLLD 368
+// against 338 us, GLM 211 against 202)
 template <int D, int BX, int BY, typename TW, bool HD = false, bool GLM = false, typename TP = TW>
 __device__ __forceinline__ void flux_tile(const Params &P, const TW *__restrict__ W, TW *__restrict__ F,
                                           int bx, int by, int bz, int tx, int ty, TW *sW, TW *sP,
